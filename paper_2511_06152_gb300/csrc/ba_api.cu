@@ -148,6 +148,7 @@ struct ba_ctx {
   std::atomic<uint64_t> launches{0};
   std::mutex api_mu;  // cluster table, plans, budget; never held across a serving round
   cudaMemPool_t pool = nullptr;  // device memory of clusters and plans (stream-ordered)
+  cudaMemPool_t scratch = nullptr;  // device scratch of single calls (scratch_alloc)
 
   // serving
   std::mutex sv_mu;
@@ -320,6 +321,30 @@ void copy_out(const std::vector<HostCopy>& items, int max_threads) {
 // round.  The pool keeps what it has reserved (no release threshold).
 cudaError_t pool_alloc(ba_ctx* ctx, void** p, size_t bytes, cudaStream_t st) {
   return cudaMallocFromPoolAsync(p, bytes, ctx->pool, st);
+}
+
+// Device scratch of one call, on the context's stream, from a pool of its own
+// that keeps up to kScratchKeep bytes between calls.  The device's default pool
+// gives its memory back at every synchronisation, so that each call mapped it
+// anew: ba_get_state of one cluster took 290 us, of which its kernel and copies
+// are 20.  Apart from the clusters' pool, so that no creation is handed (and
+// ordered behind) memory a solve's stream still uses.
+constexpr uint64_t kScratchKeep = (uint64_t)64 << 20;
+cudaError_t scratch_alloc(ba_ctx* ctx, void** p, size_t bytes) {
+  return cudaMallocFromPoolAsync(p, bytes, ctx->scratch, ctx->stream);
+}
+
+// Whether a kernel on the context's device may write doubles straight to p:
+// device memory of that device, aligned.
+bool direct_output(const ba_ctx* ctx, const double* p) {
+  if (!p) return true;
+  if ((reinterpret_cast<uintptr_t>(p) & 7) != 0) return false;
+  cudaPointerAttributes a{};
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeDevice && a.device == ctx->device;
 }
 
 bool tune_in_range(const ba_tune& t, bool mixed, std::string* why) {
@@ -694,7 +719,7 @@ ba_status run_and_collect(ba_ctx* ctx, const std::vector<ba_cluster_id>& ids, in
   StepRec* dtrace = nullptr;
   const int tcap = std::min(iters, kTraceCap);
   if (trace && tcap > 0) {
-    CUDA_TRY(ctx, cudaMallocAsync((void**)&dtrace, sizeof(StepRec) * (size_t)n * tcap, ctx->stream));
+    CUDA_TRY(ctx, scratch_alloc(ctx, (void**)&dtrace, sizeof(StepRec) * (size_t)n * tcap));
   }
   launch_gather(p->bv, tcap, p->lm_out, dtrace, ctx->stream);
   // The results go to pageable host memory, a copy that waits on the host
@@ -1996,7 +2021,7 @@ ba_status warm_copy(ba_ctx* ctx, Cluster* c, Cluster* src, const int32_t* cam_ma
   // no camera or point is shared
   int2* dp = nullptr;
   if (!pairs.empty()) {
-    CUDA_TRY(ctx, cudaMallocAsync((void**)&dp, sizeof(int2) * pairs.size(), ctx->stream));
+    CUDA_TRY(ctx, scratch_alloc(ctx, (void**)&dp, sizeof(int2) * pairs.size()));
     CUDA_TRY(ctx, cudaMemcpyAsync(dp, pairs.data(), sizeof(int2) * pairs.size(), cudaMemcpyHostToDevice, ctx->stream));
   }
   launch_warm_copy(c->d_desc, src->d_desc, dp, n_cam_pairs, dp ? dp + n_cam_pairs : nullptr,
@@ -2358,13 +2383,16 @@ BA_API ba_status ba_init(ba_ctx** out, const ba_config* cfg) {
   props.allocType = cudaMemAllocationTypePinned;
   props.location.type = cudaMemLocationTypeDevice;
   props.location.id = cfg->device;
-  const uint64_t keep = UINT64_MAX;
+  const uint64_t keep = UINT64_MAX, keep_scratch = kScratchKeep;
   if (cudaStreamCreateWithFlags(&ctx->sched_stream, cudaStreamNonBlocking) != cudaSuccess ||
       cudaStreamCreateWithFlags(&ctx->plan_stream, cudaStreamNonBlocking) != cudaSuccess ||
       cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking) != cudaSuccess ||
       cudaMemPoolCreate(&ctx->pool, &props) != cudaSuccess ||
-      cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, (void*)&keep) != cudaSuccess) {
+      cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, (void*)&keep) != cudaSuccess ||
+      cudaMemPoolCreate(&ctx->scratch, &props) != cudaSuccess ||
+      cudaMemPoolSetAttribute(ctx->scratch, cudaMemPoolAttrReleaseThreshold, (void*)&keep_scratch) != cudaSuccess) {
     if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
+    if (ctx->scratch) cudaMemPoolDestroy(ctx->scratch);
     if (ctx->sched_stream) cudaStreamDestroy(ctx->sched_stream);
     if (ctx->plan_stream) cudaStreamDestroy(ctx->plan_stream);
     if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
@@ -2440,7 +2468,7 @@ BA_API ba_status ba_transition(ba_ctx* ctx, ba_cluster_id dst, ba_cluster_id src
   }
   if (pairs.empty()) return BA_OK;
   int2* dp = nullptr;
-  CUDA_TRY(ctx, cudaMallocAsync((void**)&dp, sizeof(int2) * pairs.size(), ctx->stream));
+  CUDA_TRY(ctx, scratch_alloc(ctx, (void**)&dp, sizeof(int2) * pairs.size()));
   CUDA_TRY(ctx, cudaMemcpyAsync(dp, pairs.data(), sizeof(int2) * pairs.size(), cudaMemcpyHostToDevice, ctx->stream));
   launch_transition(c->d_desc, s->d_desc, dp, (int)pairs.size(), ctx->stream);
   launch_camreal(one_view(c->d_desc, c->nf), ctx->mixed, ctx->stream);  // camera records of the new poses
@@ -2468,7 +2496,7 @@ BA_API ba_status ba_footprints(ba_ctx* ctx, int32_t n, const double* intr, doubl
   const size_t b_in = sizeof(double) * (size_t)n * (7 + 9 + 3), b_h = sizeof(double) * nh,
                b_out = sizeof(double) * (size_t)n * 12;
   char* buf = nullptr;
-  CUDA_TRY(ctx, cudaMallocAsync((void**)&buf, b_in + b_h + b_out, ctx->stream));
+  CUDA_TRY(ctx, scratch_alloc(ctx, (void**)&buf, b_in + b_h + b_out));
   double* d_intr = (double*)buf;
   double* d_R = d_intr + 7 * (size_t)n;
   double* d_T = d_R + 9 * (size_t)n;
@@ -2502,7 +2530,7 @@ BA_API ba_status ba_patch_transfer_poses(ba_ctx* ctx, int32_t n, const double* p
   const size_t np0 = 2 * (size_t)n, ncam = 19, nk = 19 * (size_t)m, nout = 2 * (size_t)n * m;
   const size_t bytes = sizeof(double) * (np0 + ncam + nk + nout) + (inside ? (size_t)n * m : 0);
   char* buf = nullptr;
-  CUDA_TRY(ctx, cudaMallocAsync((void**)&buf, bytes, ctx->stream));
+  CUDA_TRY(ctx, scratch_alloc(ctx, (void**)&buf, bytes));
   // the double2 arrays (centres in and out) first, at even offsets of the
   // allocation's 256-byte aligned start
   double* d_p0 = (double*)buf;
@@ -2541,7 +2569,7 @@ BA_API ba_status ba_patch_transfer_planar(ba_ctx* ctx, int32_t n, const double* 
   std::lock_guard<std::mutex> gl(ctx->api_mu);
   const size_t nq = 2 * (size_t)n, nout = 2 * (size_t)n * m;
   char* buf = nullptr;
-  CUDA_TRY(ctx, cudaMallocAsync((void**)&buf, sizeof(double) * (nq + 3 * (size_t)m + nout), ctx->stream));
+  CUDA_TRY(ctx, scratch_alloc(ctx, (void**)&buf, sizeof(double) * (nq + 3 * (size_t)m + nout)));
   // the double2 arrays (centres, displacements, output) first, at even offsets
   double* d_q0 = (double*)buf;
   double* d_g = d_q0 + nq;
@@ -2569,7 +2597,7 @@ BA_API ba_status ba_footprint_overlaps(ba_ctx* ctx, int32_t na, const double* qa
   const size_t ba_ = sizeof(double) * 12 * (size_t)na, bb = sizeof(double) * 12 * (size_t)nb,
                bo = sizeof(double) * (size_t)na * nb;
   char* buf = nullptr;
-  CUDA_TRY(ctx, cudaMallocAsync((void**)&buf, ba_ + bb + bo, ctx->stream));
+  CUDA_TRY(ctx, scratch_alloc(ctx, (void**)&buf, ba_ + bb + bo));
   double* d_a = (double*)buf;
   double* d_b = d_a + 12 * (size_t)na;
   double* d_o = d_b + 12 * (size_t)nb;
@@ -2839,8 +2867,16 @@ BA_API ba_status ba_get_state(ba_ctx* ctx, ba_cluster_id id, double* R, double* 
   // destinations get it through one copy into pinned staging
   const size_t nr = (size_t)c->nc * 9, nt = (size_t)c->nc * 3, nx = (size_t)c->np * 3;
   const size_t total = nr + nt + nx;
+  // device destinations the kernel can write itself get the state with no
+  // block and no copies between
+  if (ptr_kind == BA_PTR_DEVICE && direct_output(ctx, R) && direct_output(ctx, T) && direct_output(ctx, X)) {
+    launch_export_state(c->d_desc, c->h, ctx->mixed, R, T, nx ? X : nullptr, ctx->stream);
+    note_direct(ctx);
+    CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
+    return BA_OK;
+  }
   double* tmp = nullptr;
-  CUDA_TRY(ctx, cudaMallocAsync((void**)&tmp, sizeof(double) * total, ctx->stream));
+  CUDA_TRY(ctx, scratch_alloc(ctx, (void**)&tmp, sizeof(double) * total));
   launch_export_state(c->d_desc, c->h, ctx->mixed, R ? tmp : nullptr, T ? tmp + nr : nullptr,
                       X && nx ? tmp + nr + nt : nullptr, ctx->stream);
   note_direct(ctx);
@@ -2915,7 +2951,7 @@ BA_API ba_status ba_get_state_batch(ba_ctx* ctx, const ba_cluster_id* ids, int32
       ctx->hstage_bytes = want;
     }
     double* tmp = nullptr;
-    CUDA_TRY(ctx, cudaMallocAsync((void**)&tmp, sizeof(double) * total, ctx->stream));
+    CUDA_TRY(ctx, scratch_alloc(ctx, (void**)&tmp, sizeof(double) * total));
     size_t off = 0;
     for (int i = i0; i < i1; ++i) {
       const Cluster* c = cs[i];
@@ -2954,7 +2990,7 @@ BA_API ba_status ba_reprojection_errors(ba_ctx* ctx, ba_cluster_id id, double* e
   if (!c) return BA_ERR_NOT_FOUND;
   if (c->no == 0) return BA_OK;
   double* d = nullptr;
-  CUDA_TRY(ctx, cudaMallocAsync((void**)&d, sizeof(double) * c->no, ctx->stream));
+  CUDA_TRY(ctx, scratch_alloc(ctx, (void**)&d, sizeof(double) * c->no));
   launch_reproj(c->d_desc, c->h, ctx->mixed, d, ctx->stream);
   note_direct(ctx);
   std::vector<double> pmv(c->no);
@@ -3164,7 +3200,7 @@ BA_API ba_status ba_probe_fp32_fma(ba_ctx* ctx, int32_t ctas_per_sm, int32_t ite
   CUDA_TRY(ctx, cudaSetDevice(ctx->device));
   float* sink = nullptr;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
-  CUDA_TRY(ctx, cudaMallocAsync((void**)&sink, sizeof(float), ctx->stream));
+  CUDA_TRY(ctx, scratch_alloc(ctx, (void**)&sink, sizeof(float)));
   CUDA_TRY(ctx, cudaEventCreate(&e0));
   CUDA_TRY(ctx, cudaEventCreate(&e1));
   const int ctas = ctas_per_sm * num_sms();
@@ -3230,6 +3266,7 @@ BA_API ba_status ba_shutdown(ba_ctx* ctx) {
   }
   cudaStreamSynchronize(ctx->stream);
   cudaMemPoolDestroy(ctx->pool);
+  cudaMemPoolDestroy(ctx->scratch);
   cudaStreamDestroy(ctx->sched_stream);
   cudaStreamDestroy(ctx->plan_stream);
   cudaStreamDestroy(ctx->copy_stream);
