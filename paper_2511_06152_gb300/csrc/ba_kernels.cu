@@ -864,11 +864,13 @@ __global__ void __launch_bounds__(kChunkThreads, MIXED ? kLinSchurMinBlocksMixed
 // to ~2^-48 of the total; binary64 adds run at 1/59 of the binary32 rate),
 // or of binary64 partials in binary64.
 struct AccF {
+  using Raw = dfl;
   dfl v{0.f, 0.f};
   __device__ __forceinline__ void add(float x) { v = df_add_f(v, x); }
   __device__ __forceinline__ double get() const { return (double)v.hi + (double)v.lo; }
 };
 struct AccD {
+  using Raw = double;
   double v = 0.0;
   __device__ __forceinline__ void add(double x) { v += x; }
   __device__ __forceinline__ double get() const { return v; }
@@ -876,56 +878,128 @@ struct AccD {
 template <typename Real> struct AccOf { using T = AccD; };
 template <> struct AccOf<float> { using T = AccF; };
 
-// Item `it` of a cluster (a free camera, it < n_free, or a camera pair): sum
-// its chunk partials in chunk order, by one warp (lane i owns element i and
-// i + 32), into camsum / pairsum.
+__device__ __forceinline__ AccF acc_join(AccF a, AccF b) { return AccF{df_add(a.v, b.v)}; }
+__device__ __forceinline__ AccD acc_join(AccD a, AccD b) { return AccD{a.v + b.v}; }
+
+// Every free camera and camera pair ("item") of the batch's clusters: its
+// chunk partials, added, into camsum / pairsum.
+//
+// Per iteration on GB300: one cluster of 235 k observations 39 -> 12 us (97 ->
+// 18 in binary64), 12 clusters 25 -> 17, 400 images 24 -> 27, 128 clusters
+// 68 -> 76 (their short lists filled the GPU as a warp each too).
+//
+// What bounds it is the latency of the loads: an item is a list of rows, up
+// to one per chunk of the cluster (501 of them for 235 k observations), and
+// one warp per item added them a few at a time, 39 us per iteration of that
+// single cluster (97 us in binary64) with most of the GPU idle.  A CTA has
+// kRedSegs groups of kCamPart lanes (lane = element of the row).  A list of
+// up to kRedLong rows is one group's; a longer one is cut into kRedSegs
+// contiguous runs, a group each, whose sums are joined in order.  Eight rows
+// are in flight per lane.  The cut depends on the list's length alone, so a
+// cluster's sums are the same alone and in any batch.  With more items than
+// CTAs, a CTA takes several items at a time, a grid apart (a cluster's long
+// lists, its images', are neighbours), and their short lists run side by side.
+constexpr int kRedSegs = 6;
+constexpr int kRedLong = 48;
+constexpr int kRedThreads = 256;
+constexpr int kRedCtasPerSm = 8;
+static_assert(kRedSegs * kCamPart <= kRedThreads && kPairPart <= kCamPart, "a group of lanes per row");
+
+// rows [p, p1) of a list, element el, in order
 template <typename Real>
-__device__ __forceinline__ void reduce_item_partials(const DevCluster& C, int it, int lane) {
-  using Acc = typename AccOf<Real>::T;
-  const bool cam = it < C.n_free;
-  const int key = cam ? it : it - C.n_free;
-  const int width = cam ? 39 : 36, stride = cam ? kCamPart : kPairPart;
-  const int* slots = cam ? C.cam_slots : C.pair_slots;
-  const int b = cam ? C.cam_slot_begin[key] : C.pair_slot_begin[key];
-  const int e = cam ? C.cam_slot_begin[key + 1] : C.pair_slot_begin[key + 1];
-  const Real* part = (const Real*)(cam ? C.campart : C.pairpart);
-  double* out = cam ? C.camsum + (size_t)kCamPart * key : C.pairsum + (size_t)kPairPart * key;
-  const bool two = lane + 32 < width;
-  Acc v0, v1;
-  int p = b;
-  for (; p + 4 <= e; p += 4) {  // four independent loads in flight, added in slot order
-    const Real* a0 = part + (size_t)stride * slots[p];
-    const Real* a1 = part + (size_t)stride * slots[p + 1];
-    const Real* a2 = part + (size_t)stride * slots[p + 2];
-    const Real* a3 = part + (size_t)stride * slots[p + 3];
-    const Real x0 = lane < width ? a0[lane] : Real(0), x1 = lane < width ? a1[lane] : Real(0);
-    const Real x2 = lane < width ? a2[lane] : Real(0), x3 = lane < width ? a3[lane] : Real(0);
-    const Real y0 = two ? a0[lane + 32] : Real(0), y1 = two ? a1[lane + 32] : Real(0);
-    const Real y2 = two ? a2[lane + 32] : Real(0), y3 = two ? a3[lane + 32] : Real(0);
-    v0.add(x0); v0.add(x1); v0.add(x2); v0.add(x3);
-    v1.add(y0); v1.add(y1); v1.add(y2); v1.add(y3);
+__device__ __forceinline__ typename AccOf<Real>::T add_rows(const Real* part, int stride, const int* slots, int p,
+                                                            int p1) {
+  typename AccOf<Real>::T acc;
+  for (; p + 8 <= p1; p += 8) {
+    Real x[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) x[i] = part[(size_t)stride * slots[p + i]];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) acc.add(x[i]);
   }
-  for (; p < e; ++p) {
-    const Real* a0 = part + (size_t)stride * slots[p];
-    if (lane < width) v0.add(a0[lane]);
-    if (two) v1.add(a0[lane + 32]);
+  if (p < p1) {  // the last rows, all loads before the adds as well
+    Real x[7];
+#pragma unroll
+    for (int i = 0; i < 7; ++i) x[i] = p + i < p1 ? part[(size_t)stride * slots[p + i]] : Real(0);
+#pragma unroll
+    for (int i = 0; i < 7; ++i)
+      if (p + i < p1) acc.add(x[i]);
   }
-  if (lane < width) out[lane] = v0.get();
-  if (two) out[lane + 32] = v1.get();
+  return acc;
 }
 
-// Warp per free camera or camera pair of every cluster of the batch.
+// an item's list and where its sums go
+struct RedItem {
+  const int* slots;
+  const void* part;
+  double* out;
+  int begin, n, width;  // n = 0: nothing to do (its cluster is inactive, or no such item)
+};
+__device__ __forceinline__ RedItem red_item(const BatchView& bv, int g) {
+  const int s = find_slot(bv.item_pre, bv.n, g);
+  const DevCluster& C = bv.cl[s];
+  if (!C.lm->active) return RedItem{};
+  const int it = g - bv.item_pre[s];
+  const bool cam = it < C.n_free;
+  const int key = cam ? it : it - C.n_free;
+  const int* begin = (cam ? C.cam_slot_begin : C.pair_slot_begin) + key;
+  RedItem r;
+  r.begin = begin[0];
+  r.n = begin[1] - r.begin;
+  r.slots = cam ? C.cam_slots : C.pair_slots;
+  r.part = cam ? C.campart : C.pairpart;
+  r.out = cam ? C.camsum + (size_t)kCamPart * key : C.pairsum + (size_t)kPairPart * key;
+  r.width = cam ? 39 : 36;
+  return r;
+}
+
 template <typename Real>
-__global__ void __launch_bounds__(256) k_partial_reduce(BatchView bv) {
-  const int lane = threadIdx.x & 31;
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int nwarps = (gridDim.x * blockDim.x) >> 5;
+__global__ void __launch_bounds__(kRedThreads) k_partial_reduce(BatchView bv) {
+  using Acc = typename AccOf<Real>::T;
+  __shared__ typename Acc::Raw sums[2][kRedSegs][kCamPart];  // two items' worth: one barrier per long item
+  __shared__ RedItem items[kRedSegs];
+  const int seg = threadIdx.x / kCamPart, el = threadIdx.x - seg * kCamPart;
   const int total = bv.tot[2];
-  for (int g = warp; g < total; g += nwarps) {
-    const int s = find_slot(bv.item_pre, bv.n, g);
-    const DevCluster& C = bv.cl[s];
-    if (!C.lm->active) continue;
-    reduce_item_partials<Real>(C, g - bv.item_pre[s], lane);
+  // items a CTA takes at a time: as many as spread the batch over the grid in one round, at most one per group
+  const int group = min(kRedSegs, (total + (int)gridDim.x - 1) / (int)gridDim.x);
+  int buf = 0;
+  for (int g0 = blockIdx.x; g0 < total; g0 += gridDim.x * group) {
+    if (threadIdx.x < group) {
+      const int g = g0 + threadIdx.x * gridDim.x;
+      RedItem r{};
+      if (g < total) r = red_item(bv, g);
+      items[threadIdx.x] = r;
+    }
+    __syncthreads();
+    if (seg < group) {  // the short lists, a group each
+      const RedItem r = items[seg];
+      if (r.n > 0 && r.n <= kRedLong && el < r.width) {
+        const Real* part = (const Real*)r.part + el;
+        const int stride = r.width == 36 ? kPairPart : kCamPart;
+        r.out[el] = add_rows<Real>(part, stride, r.slots, r.begin, r.begin + r.n).get();
+      }
+    }
+    for (int i = 0; i < group; ++i) {  // the long ones, all groups together
+      const RedItem r = items[i];
+      if (r.n <= kRedLong) continue;
+      const bool live = seg < kRedSegs && el < r.width;
+      if (live) {
+        const Real* part = (const Real*)r.part + el;
+        const int stride = r.width == 36 ? kPairPart : kCamPart;
+        const int per = (r.n + kRedSegs - 1) / kRedSegs;
+        const int p0 = r.begin + seg * per, p1 = r.begin + min(r.n, (seg + 1) * per);
+        sums[buf][seg][el] = add_rows<Real>(part, stride, r.slots, p0, p1).v;
+      }
+      __syncthreads();
+      if (seg == 0 && live) {
+        Acc t{sums[buf][0][el]};
+#pragma unroll
+        for (int q = 1; q < kRedSegs; ++q) t = acc_join(t, Acc{sums[buf][q][el]});
+        r.out[el] = t.get();
+      }
+      buf ^= 1;
+    }
+    __syncthreads();  // items[] is read no more
   }
 }
 
@@ -2360,7 +2434,7 @@ static void launch_lin_schur(const BatchView& bv, int diag, cudaStream_t st) {
 template <bool MIXED>
 static void launch_partial_reduce(const BatchView& bv, cudaStream_t st) {
   using Real = typename RealOf<MIXED>::T;
-  LAUNCH(KK_PARTIAL_REDUCE, st, k_partial_reduce<Real><<<grid_for(bv.total_items, 8, num_sms() * 16), 256, 0, st>>>(bv));
+  LAUNCH(KK_PARTIAL_REDUCE, st, k_partial_reduce<Real><<<grid_for(bv.total_items, 1, num_sms() * kRedCtasPerSm), kRedThreads, 0, st>>>(bv));
 }
 
 template <bool MIXED>
