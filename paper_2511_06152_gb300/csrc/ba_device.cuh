@@ -301,86 +301,140 @@ __device__ __forceinline__ bool obs_linearize(const Real* Rm, Real dx, Real dy, 
   return true;
 }
 
-// The LM decision of one cluster, by one warp, once every tile of its
-// back-substitution is done: F(x + d) and pred from the tiles' partial sums
-// (in k_cost_init's summation order), the gain ratio,
-// accept or reject, Nielsen's update of mu and nu, the step record; on
-// acceptance in binary64 the camera records of the new state.
-template <bool MIXED>
-__device__ __forceinline__ void lm_update_warp(const DevCluster& C, int lane) {
+// The LM decision of one cluster once every tile of its back-substitution is
+// done, by one thread: gain ratio from F(x + d) and pred (Fo, pp: the sums of
+// the tiles' cost and pred terms), accept or reject, Nielsen's update of mu and
+// nu, the step record.  Returns 1 when the step was accepted.
+__device__ __forceinline__ int lm_decide(const DevCluster& C, double Fo, double pp) {
   LmState* lm = C.lm;
   const bool ok = lm->status == 0;
+  const double F = lm->F;
+  const double Fn = ok ? Fo + lm->prior_new : F;
+  const double pred = ok ? 0.5 * (pp + lm->pred_cam) : 0.0;
+  const double gain = pred > 0.0 ? (F - Fn) / pred : 0.0;
+  const int accepted = ok && pred > 0.0 && gain > 0.0;
+  const double mu_used = lm->mu;
+  if (accepted) {
+    const double tt = 2.0 * gain - 1.0;
+    const double fct = 1.0 - tt * tt * tt;
+    lm->mu = mu_used * (fct > 1.0 / 3.0 ? fct : 1.0 / 3.0);
+    lm->nu = 2.0;
+    lm->cur ^= 1;
+    lm->F = Fn;
+    lm->n_accepted += 1;
+  } else {
+    lm->mu = mu_used * lm->nu;
+    lm->nu *= 2.0;
+  }
+  if (C.trace_cap > 0) {
+    StepRec& r = C.trace[lm->iter % C.trace_cap];
+    r.accepted = accepted;
+    r.status = lm->status;
+    r.F_before = F;
+    r.F_after = Fn;
+    r.predicted = pred;
+    r.gain = gain;
+    r.mu_used = mu_used;
+    r.mu = lm->mu;
+    r.nu = lm->nu;
+  }
+  lm->iter += 1;
+  if (lm->iter >= lm->iters_target) lm->active = 0;
+  // converged (serving): an accepted step, not the first since arming, that
+  // lowered F by at most ftol * F
+  if (lm->ftol > 0.0 && accepted && lm->iter - lm->iter0 >= 2 && F - Fn <= lm->ftol * F) lm->active = 0;
+  lm->pt_fail = 0;
+  lm->mu_f = (float)lm->mu;
+  return accepted;
+}
+
+// binary64 path: the camera records of an accepted step's state (buffer cur),
+// by nt threads, t = 0 .. nt - 1
+__device__ __forceinline__ void refresh_camreal(const DevCluster& C, int cur, int t, int nt) {
+  double* cr = (double*)C.camreal;
+  for (int k = t; k < C.n_cams; k += nt) {
+    const double* R = C.R + ((size_t)cur * C.n_cams + k) * 9;
+    const double* T = C.T + ((size_t)cur * C.n_cams + k) * 3;
+    double* o = cr + (size_t)kCamReal * k;
+    for (int i = 0; i < 9; ++i) o[i] = R[i];
+    for (int i = 0; i < 3; ++i) o[9 + i] = T[i];
+  }
+}
+
+// The tiles' sums are formed in the order of k_cost_init (kCostInitThreads
+// threads, thread t of warp t / 32 adds tiles t, t + 256, ... in turn; a warp
+// tree; the 8 warps in order), so that F carried from one iteration to the
+// next equals F evaluated afresh at the start of a solve, bit for bit.
+__device__ __forceinline__ void lm_tile_run(const DevCluster& C, int first, double& a, double& b) {
+  const double2* tp = reinterpret_cast<const double2*>(C.tilepart);
+  a = b = 0.0;
+  int i = first;
+  for (; i + 3 * kCostInitThreads < C.n_tiles; i += 4 * kCostInitThreads) {  // four loads in flight
+    double2 v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q] = __ldcg(tp + i + q * kCostInitThreads);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      a += v[q].x;
+      b += v[q].y;
+    }
+  }
+  for (; i < C.n_tiles; i += kCostInitThreads) {
+    const double2 v = __ldcg(tp + i);
+    a += v.x;
+    b += v.y;
+  }
+  a = warp_sum(a);
+  b = warp_sum(b);
+}
+
+// the whole step by one warp
+template <bool MIXED>
+__device__ __forceinline__ void lm_update_warp(const DevCluster& C, int lane) {
   double Fo = 0.0, pp = 0.0;
-  if (ok) {
-    // the order of k_cost_init's sum over a 256-thread CTA (thread t of warp
-    // t / 32 adds tiles t, t + 256, ... in turn; a warp tree; the 8 warps in
-    // order), so that F carried from one iteration to the next equals F
-    // evaluated afresh at the start of a solve, bit for bit
-    const double2* tp = reinterpret_cast<const double2*>(C.tilepart);
+  if (C.lm->status == 0) {
     for (int w = 0; w < kCostInitThreads / 32; ++w) {
-      double a = 0.0, b = 0.0;
-      for (int i = 32 * w + lane; i < C.n_tiles; i += kCostInitThreads) {
-        const double2 v = tp[i];
-        a += v.x;
-        b += v.y;
-      }
-      Fo += warp_sum(a);
-      pp += warp_sum(b);
+      double a, b;
+      lm_tile_run(C, 32 * w + lane, a, b);
+      Fo += a;
+      pp += b;
     }
   }
-  int accepted = 0, cur = 0;
-  if (lane == 0) {
-    const double F = lm->F;
-    const double Fn = ok ? Fo + lm->prior_new : F;
-    const double pred = ok ? 0.5 * (pp + lm->pred_cam) : 0.0;
-    const double gain = pred > 0.0 ? (F - Fn) / pred : 0.0;
-    accepted = ok && pred > 0.0 && gain > 0.0;
-    const double mu_used = lm->mu;
-    if (accepted) {
-      const double tt = 2.0 * gain - 1.0;
-      const double fct = 1.0 - tt * tt * tt;
-      lm->mu = mu_used * (fct > 1.0 / 3.0 ? fct : 1.0 / 3.0);
-      lm->nu = 2.0;
-      lm->cur ^= 1;
-      lm->F = Fn;
-      lm->n_accepted += 1;
-    } else {
-      lm->mu = mu_used * lm->nu;
-      lm->nu *= 2.0;
-    }
-    if (C.trace_cap > 0) {
-      StepRec& r = C.trace[lm->iter % C.trace_cap];
-      r.accepted = accepted;
-      r.status = lm->status;
-      r.F_before = F;
-      r.F_after = Fn;
-      r.predicted = pred;
-      r.gain = gain;
-      r.mu_used = mu_used;
-      r.mu = lm->mu;
-      r.nu = lm->nu;
-    }
-    lm->iter += 1;
-    if (lm->iter >= lm->iters_target) lm->active = 0;
-    // converged (serving): an accepted step, not the first since arming, that
-    // lowered F by at most ftol * F
-    if (lm->ftol > 0.0 && accepted && lm->iter - lm->iter0 >= 2 && F - Fn <= lm->ftol * F) lm->active = 0;
-    lm->pt_fail = 0;
-    lm->mu_f = (float)lm->mu;
-    cur = lm->cur;
-  }
+  int accepted = lane == 0 ? lm_decide(C, Fo, pp) : 0;
   accepted = __shfl_sync(BA_FULL_MASK, accepted, 0);
-  cur = __shfl_sync(BA_FULL_MASK, cur, 0);
-  if (!MIXED && accepted) {  // refresh the binary64 camera records for the new state
-    double* cr = (double*)C.camreal;
-    for (int k = lane; k < C.n_cams; k += 32) {
-      const double* R = C.R + ((size_t)cur * C.n_cams + k) * 9;
-      const double* T = C.T + ((size_t)cur * C.n_cams + k) * 3;
-      double* o = cr + (size_t)kCamReal * k;
-      for (int i = 0; i < 9; ++i) o[i] = R[i];
-      for (int i = 0; i < 3; ++i) o[9 + i] = T[i];
+  if (!MIXED && accepted) refresh_camreal(C, __shfl_sync(BA_FULL_MASK, lane == 0 ? C.lm->cur : 0, 0), lane, 32);
+}
+
+// the whole step by a CTA of kCostInitThreads threads (red: shared [2][8] and
+// one more double)
+template <bool MIXED>
+__device__ __forceinline__ void lm_update_cta(const DevCluster& C, double* red) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  constexpr int nw = kCostInitThreads / 32;
+  if (C.lm->status == 0) {
+    double a, b;
+    lm_tile_run(C, threadIdx.x, a, b);
+    if (lane == 0) {
+      red[wid] = a;
+      red[nw + wid] = b;
     }
+  } else if (lane == 0) {
+    red[wid] = red[nw + wid] = 0.0;
   }
+  __syncthreads();
+  int* acc = reinterpret_cast<int*>(red + 2 * nw);
+  if (threadIdx.x == 0) {
+    double Fo = 0.0, pp = 0.0;
+    for (int w = 0; w < nw; ++w) {
+      Fo += red[w];
+      pp += red[nw + w];
+    }
+    acc[0] = lm_decide(C, Fo, pp);
+    acc[1] = C.lm->cur;
+  }
+  __syncthreads();
+  if (!MIXED && acc[0]) refresh_camreal(C, acc[1], threadIdx.x, kCostInitThreads);
+  __syncthreads();  // red is free
 }
 
 }  // namespace bagpu

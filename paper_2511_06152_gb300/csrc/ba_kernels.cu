@@ -1773,25 +1773,32 @@ __global__ void __launch_bounds__(kFactorThreads) k_factor_solve(BatchView bv, i
 template <bool MIXED>
 __device__ void backsub_tile(const DevCluster& C, LmState* lm, int local, int lane);
 
-// add a warp's count of finished tiles to its cluster's total; the warp that
-// completes the total takes the cluster's LM decision
-template <bool MIXED>
-__device__ __forceinline__ void publish_tiles(const DevCluster& C, int count, int lane) {
+// add a warp's count of finished tiles to its cluster's total; true for the
+// warp that completes the total: the cluster's LM step is due
+__device__ __forceinline__ bool publish_tiles(const DevCluster& C, int count, int lane) {
   int done = 0;
   if (lane == 0) {
     __threadfence();  // this warp's partial sums before the count
     done = atomicAdd(&C.lm->tiles_done, count) + count;
   }
   done = __shfl_sync(BA_FULL_MASK, done, 0);
-  if (done == C.n_tiles) {
-    __threadfence();
-    lm_update_warp<MIXED>(C, lane);
-  }
+  if (done != C.n_tiles) return false;
+  __threadfence();
+  return true;
 }
 
+// Clusters that a CTA's warps complete get their LM step from the whole CTA at
+// its end (the sums over a single cluster's 8,000 tiles took one warp 40 of
+// the kernel's 62 us); past this many, from the completing warp itself.
+constexpr int kMaxDue = 64;
+
 template <bool MIXED>
-__global__ void __launch_bounds__(256) k_backsub_cost(BatchView bv) {
+__global__ void __launch_bounds__(kCostInitThreads) k_backsub_cost(BatchView bv) {
   using Real = typename RealOf<MIXED>::T;
+  __shared__ int due[kMaxDue], n_due;
+  __shared__ double red[2 * (kCostInitThreads / 32) + 1];
+  if (threadIdx.x == 0) n_due = 0;
+  __syncthreads();
   const int lane = threadIdx.x & 31;
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -1799,15 +1806,22 @@ __global__ void __launch_bounds__(256) k_backsub_cost(BatchView bv) {
   // each warp takes a contiguous run of tiles, so that its tiles mostly
   // belong to one cluster: it counts them per cluster and publishes the
   // count once per cluster it leaves (one fence and one atomic each); the
-  // warp whose count completes a cluster takes the cluster's LM decision,
-  // every other tile's partial sums being written by then
+  // warp whose count completes a cluster, every other tile's partial sums
+  // being written by then, hands the cluster's LM step to its CTA
   const int per = (total + nwarps - 1) / nwarps;
   const int g0 = warp * per, g1 = min(total, g0 + per);
   int s = g0 < g1 ? find_slot(bv.tile_pre, bv.n, g0) : 0;
   int pending = 0;
+  auto leave = [&](int slot) {
+    if (!pending || !publish_tiles(bv.cl[slot], pending, lane)) return;
+    int at = lane == 0 ? atomicAdd(&n_due, 1) : 0;
+    at = __shfl_sync(BA_FULL_MASK, at, 0);
+    if (at >= kMaxDue) lm_update_warp<MIXED>(bv.cl[slot], lane);
+    else if (lane == 0) due[at] = slot;
+  };
   for (int g = g0; g < g1; ++g) {
     while (g >= bv.tile_pre[s + 1]) {  // the next cluster: publish the count of this one
-      if (pending) publish_tiles<MIXED>(bv.cl[s], pending, lane);
+      leave(s);
       pending = 0;
       ++s;
     }
@@ -1817,7 +1831,10 @@ __global__ void __launch_bounds__(256) k_backsub_cost(BatchView bv) {
     if (lm->status == 0) backsub_tile<MIXED>(C, lm, g - bv.tile_pre[s], lane);
     ++pending;
   }
-  if (pending) publish_tiles<MIXED>(bv.cl[s], pending, lane);
+  leave(s);
+  __syncthreads();
+  const int n = min(n_due, kMaxDue);
+  for (int i = 0; i < n; ++i) lm_update_cta<MIXED>(bv.cl[due[i]], red);
 }
 
 // back-substitution and candidate cost of one tile (one warp)
@@ -2447,7 +2464,7 @@ static void launch_iteration_t(const BatchView& bv, int refine_steps, cudaStream
          k_factor_solve<MIXED><<<grid_for(bv.n, 1, 65535), bv.factor_threads, smem, st>>>(bv, refine_steps, 0));
   if (big)
     for (const BigRef& b : *big) launch_big_solve(b, MIXED, refine_steps, 0, st);
-  LAUNCH(KK_BACKSUB, st, k_backsub_cost<MIXED><<<grid_for(bv.total_tiles, 8, sms * bv.back_ctas_per_sm), 256, 0, st>>>(bv));
+  LAUNCH(KK_BACKSUB, st, k_backsub_cost<MIXED><<<grid_for(bv.total_tiles, 8, sms * bv.back_ctas_per_sm), kCostInitThreads, 0, st>>>(bv));
 }
 
 void launch_iteration(const BatchView& bv, bool mixed, int refine_steps, cudaStream_t st,
