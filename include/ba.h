@@ -116,8 +116,8 @@ typedef struct {
  * binary64 CUDA-core factorisation instead (same envelope, same refinement),
  * for comparisons. */
 #define BA_FLAG_BIG_FP64_FACTOR 4
-/* Reduced camera systems of up to 32 free images are factored in shared
- * memory by one CTA: in binary64 in BA_FP64, in double-float on the binary32
+/* Reduced camera systems of up to 32 free images are factored in the shared
+ * memory of one thread-block cluster: in binary64 in BA_FP64, in double-float on the binary32
  * pipe in BA_MIXED (the system equilibrated by powers of two), then the
  * configured refinement passes against the binary64 S.  This flag selects
  * the double-float factorisation in BA_FP64 too, for comparisons (no effect
@@ -505,7 +505,7 @@ BA_API ba_status ba_cost_noalloc(const ba_cluster_desc* d, void* stream, double*
 /* ---- Autotuning of the launch shapes ----
  *
  * Launch and presort parameters of the LM iteration.  None changes what is
- * computed; chunk_tiles and factor_nb change the order of some sums (every
+ * computed; chunk_tiles changes the order of some sums (every
  * configuration is deterministic: alone = in a batch, bit for bit).
  * Values: chunk_tiles 0 (the precision's maximum: 16 mixed, 8 FP64) or
  * 4 .. that maximum; lin_ctas_per_sm and back_ctas_per_sm 1 .. 32;
@@ -517,8 +517,9 @@ typedef struct {
   int32_t chunk_tiles;      /* observations per linearise+Schur CTA, in tiles of up to 32 (whole points) */
   int32_t lin_ctas_per_sm;  /* linearise+Schur grid: CTAs per SM before it strides */
   int32_t back_ctas_per_sm; /* back-substitution grid: CTAs per SM before it strides */
-  int32_t factor_nb;        /* panel width of the shared-memory Cholesky (clusters of <= 32 free images) */
-  int32_t factor_threads;   /* threads of its CTA */
+  int32_t factor_nb;        /* accepted and without effect: the factor of clusters of <= 32 free images works on
+                               block columns of 8 */
+  int32_t factor_threads;   /* that factor runs on four CTAs of half as many threads (at least 192) */
   int32_t big_panel_w;      /* column-block width of the tensor-core solver's diagonal factorisation */
   int32_t batch_chains;     /* a batch's LM iterations as this many concurrent launch chains over disjoint
                                parts of the batch (clusters dealt by decreasing size); 1: one chain */

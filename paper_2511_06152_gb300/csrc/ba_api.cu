@@ -395,7 +395,6 @@ ba_tune tune_to_abi(const TuneParams& p) {
 void apply_tune(const ba_ctx* ctx, BatchView& bv) {
   bv.lin_ctas_per_sm = ctx->tune.lin_ctas_per_sm;
   bv.back_ctas_per_sm = ctx->tune.back_ctas_per_sm;
-  bv.factor_nb = ctx->tune.factor_nb;
   bv.factor_threads = ctx->tune.factor_threads;
   bv.factor_df = ctx->mixed || ctx->small_df;
 }
@@ -1711,7 +1710,7 @@ ba_status build_cluster(ba_ctx* ctx, const ba_cluster_desc* d, Cluster* c, const
   const size_t o_cpart = Lo.add(rs * kCamPart * (size_t)n_cslots);
   const size_t o_ppart = Lo.add(rs * kPairPart * (size_t)n_pslots);
   const size_t o_csum = Lo.add(sizeof(double) * kCamPart * (size_t)nf);
-  const size_t o_psum = Lo.add(sizeof(double) * kPairPart * (size_t)n_pairs);
+  const size_t o_psum = Lo.add(big ? sizeof(double) * kPairPart * (size_t)n_pairs : 0);
   const size_t o_S = Lo.add(sizeof(double) * (size_t)n * n);
   const size_t o_rhs = Lo.add(sizeof(double) * n);
   const size_t o_gc = Lo.add(sizeof(double) * n);
@@ -1916,6 +1915,8 @@ ba_status build_cluster(ba_ctx* ctx, const ba_cluster_desc* d, Cluster* c, const
   h.n_cslots = n_cslots; h.n_pslots = n_pslots;
   h.sigma_px = d->sigma_px; h.huber_delta = d->huber_delta_px; h.sigma_gnss = d->sigma_gnss_m;
   h.sigma_imu = d->sigma_imu_rad;
+  h.inv_gnss2 = d->sigma_gnss_m > 0.0 ? 1.0 / (d->sigma_gnss_m * d->sigma_gnss_m) : 0.0;
+  h.inv_imu2 = d->sigma_imu_rad > 0.0 ? 1.0 / (d->sigma_imu_rad * d->sigma_imu_rad) : 0.0;
   h.inv_sigma_f = (float)(1.0 / d->sigma_px);
   h.delta_f = (float)d->huber_delta_px;
   h.half_inv_s2_f = (float)(0.5 / (d->sigma_px * d->sigma_px));
@@ -1976,6 +1977,8 @@ ba_status build_cluster(ba_ctx* ctx, const ba_cluster_desc* d, Cluster* c, const
   h.trace_cap = kTraceCap;
   c->d_desc = (DevCluster*)(arena + o_desc);
   e = cudaMemcpyAsync(c->d_desc, &h, sizeof(DevCluster), cudaMemcpyHostToDevice, up);
+  // S of the shared-memory factor: only the co-visible pairs' blocks are ever written
+  if (e == cudaSuccess && !big) e = cudaMemsetAsync(h.S, 0, sizeof(double) * (size_t)n * n, up);
   if (e == cudaSuccess) e = cudaStreamSynchronize(up);
   if (e != cudaSuccess) return fail("cluster upload: ", e);
   cudaStreamDestroy(up);
@@ -3114,7 +3117,6 @@ BA_API ba_status ba_autotune(ba_ctx* ctx, const ba_cluster_desc* descs, int32_t 
       {&TuneParams::chunk_tiles, mixed ? std::vector<int>{12, 8} : std::vector<int>{6, 4}, false},
       {&TuneParams::lin_ctas_per_sm, {4, 2}, false},
       {&TuneParams::back_ctas_per_sm, {8, 4}, false},
-      {&TuneParams::factor_nb, {4, 16}, false},
       {&TuneParams::factor_threads, {384, 256}, false},
       {&TuneParams::big_panel_w, {2, 8}, true},
       {&TuneParams::batch_chains, {2, 8}, false},

@@ -33,23 +33,30 @@ __device__ inline void write_camdf(const DevCluster& C, int buf, int k, const do
   for (int i = 38; i < kCamDf; ++i) o[i] = 0.0f;
 }
 
-// Candidate pose of camera k for the step x (in the elimination order,
-// 6 per free image): R Exp(dtheta), T + dT in binary64, written to state
-// buffer cur ^ 1 (and its double-float record in the mixed path).  A fixed
-// camera, or any camera when fail is set, keeps its pose.  For a free camera
-// *pc = d^T (mu D d + g) of its block and *pn = its prior cost at the
-// candidate; 0 otherwise.
-template <bool MIXED>
-__device__ inline void candidate_camera(const DevCluster& C, int k, const double* x, double mu, int cur, bool fail,
-                                        double* pc, double* pn) {
+// Row q of R and entry q of T of the record; the intrinsics, the same in both
+// buffers, stay as they are
+__device__ __forceinline__ void write_camdf_row(const DevCluster& C, int buf, int k, int q, const double row[3],
+                                                double t) {
+  float* o = C.camdf + ((size_t)buf * C.n_cams + k) * kCamDf;
+  for (int i = 0; i < 3; ++i) {
+    const dfl v = df_from_d(row[i]);
+    o[3 * q + i] = v.hi;
+    o[24 + 3 * q + i] = v.lo;
+  }
+  const dfl v = df_from_d(t);
+  o[9 + q] = v.hi;
+  o[12 + q] = v.lo;
+}
+
+// Candidate pose of camera k for the step x (in the elimination order, 6 per
+// free image): R Exp(dtheta), T + dT in binary64.  A fixed camera, or any
+// camera when fail is set, keeps its pose.
+__device__ inline void candidate_pose(const DevCluster& C, int k, const double* x, int cur, bool fail, double Rn[9],
+                                      double Tn[3]) {
   const int nc = C.n_cams;
   const double* Rc = C.R + (size_t)cur * nc * 9 + 9 * k;
   const double* Tc = C.T + (size_t)cur * nc * 3 + 3 * k;
-  double* Rn = C.R + (size_t)(cur ^ 1) * nc * 9 + 9 * k;
-  double* Tn = C.T + (size_t)(cur ^ 1) * nc * 3 + 3 * k;
   const int f = C.free_idx[k];
-  *pc = 0.0;
-  *pn = 0.0;
   if (f < 0 || fail) {
     for (int i = 0; i < 9; ++i) Rn[i] = Rc[i];
     for (int i = 0; i < 3; ++i) Tn[i] = Tc[i];
@@ -60,12 +67,39 @@ __device__ inline void candidate_camera(const DevCluster& C, int k, const double
     for (int r = 0; r < 3; ++r)
       for (int c = 0; c < 3; ++c) Rn[3 * r + c] = Rc[3 * r] * E[c] + Rc[3 * r + 1] * E[3 + c] + Rc[3 * r + 2] * E[6 + c];
     for (int i = 0; i < 3; ++i) Tn[i] = Tc[i] + d[3 + i];
+  }
+}
+
+// The candidate to state buffer cur ^ 1 (and its double-float record in the
+// mixed path).
+template <bool MIXED>
+__device__ inline void store_candidate(const DevCluster& C, int k, int cur, const double* Rn, const double* Tn) {
+  const int nc = C.n_cams;
+  double* Ro = C.R + (size_t)(cur ^ 1) * nc * 9 + 9 * k;
+  double* To = C.T + (size_t)(cur ^ 1) * nc * 3 + 3 * k;
+  for (int i = 0; i < 9; ++i) Ro[i] = Rn[i];
+  for (int i = 0; i < 3; ++i) To[i] = Tn[i];
+  if constexpr (MIXED) write_camdf(C, cur ^ 1, k, Rn, Tn);
+}
+
+// Both, with, for a free camera, *pc = d^T (mu D d + g) of its block and
+// *pn = its prior cost at the candidate (0 otherwise).
+template <bool MIXED>
+__device__ inline void candidate_camera(const DevCluster& C, int k, const double* x, double mu, int cur, bool fail,
+                                        double* pc, double* pn) {
+  double Rn[9], Tn[3];
+  candidate_pose(C, k, x, cur, fail, Rn, Tn);
+  store_candidate<MIXED>(C, k, cur, Rn, Tn);
+  const int f = C.free_idx[k];
+  *pc = 0.0;
+  *pn = 0.0;
+  if (f >= 0 && !fail) {
+    const double* d = x + 6 * C.fpos[f];
     double s = 0.0;
     for (int a = 0; a < 6; ++a) s += d[a] * (mu * C.Dc[6 * f + a] * d[a] + C.gc[6 * f + a]);
     *pc = s;
     *pn = prior_terms(Rn, Tn, C.R_prior + 9 * k, C.T_prior + 3 * k, C.sigma_imu, C.sigma_gnss, nullptr, nullptr);
   }
-  if constexpr (MIXED) write_camdf(C, cur ^ 1, k, Rn, Tn);
 }
 
 }  // namespace bagpu

@@ -120,18 +120,23 @@ __device__ inline void so3_exp(const double w[3], double R[9]) {
   R[7] = b * w[1] * w[2] + a * w[0];
 }
 
-__device__ inline void so3_log(const double R[9], double w[3]) {
-  double c = 0.5 * (R[0] + R[4] + R[8] - 1.0);
+// The factor of the axial part (R - R^T)^v in the rotation vector of R, t / (2
+// sin t) for the angle t of the trace; -1 within 1e-6 of a half turn.
+__device__ __forceinline__ double log_scale(double trace) {
+  double c = 0.5 * (trace - 1.0);
   c = fmin(1.0, fmax(-1.0, c));
-  const double v0 = R[7] - R[5], v1 = R[2] - R[6], v2 = R[3] - R[1];
   const double x = 1.0 - c;
-  if (x < 0.5 * kSmallAngle2) {  // t / sin t in powers of 1 - cos t
-    const double s = 0.5 * (1.0 + x * (1.0 / 3.0 + x * (2.0 / 15.0 + x * (2.0 / 35.0 + x * (8.0 / 315.0)))));
-    w[0] = s * v0; w[1] = s * v1; w[2] = s * v2;
-    return;
-  }
+  if (x < 0.5 * kSmallAngle2)  // t / sin t in powers of 1 - cos t
+    return 0.5 * (1.0 + x * (1.0 / 3.0 + x * (2.0 / 15.0 + x * (2.0 / 35.0 + x * (8.0 / 315.0)))));
   const double t = acos(c);
-  if (t > 3.14159165358979 /* pi - 1e-6 */) {
+  return t > 3.14159165358979 ? -1.0 : t / (2.0 * sin(t));
+}
+
+__device__ inline void so3_log(const double R[9], double w[3]) {
+  const double v0 = R[7] - R[5], v1 = R[2] - R[6], v2 = R[3] - R[1];
+  const double sc = log_scale(R[0] + R[4] + R[8]);
+  if (sc < 0.0) {
+    const double t = acos(fmax(-1.0, 0.5 * (R[0] + R[4] + R[8] - 1.0)));
     // axis from the column of R + I with the largest norm
     int col = 0;
     double best = -1.0;
@@ -146,23 +151,21 @@ __device__ inline void so3_log(const double R[9], double w[3]) {
     if (ax0 * v0 + ax1 * v1 + ax2 * v2 < 0.0) { ax0 = -ax0; ax1 = -ax1; ax2 = -ax2; }
     w[0] = t * ax0; w[1] = t * ax1; w[2] = t * ax2;
   } else {
-    const double s = t / (2.0 * sin(t));
-    w[0] = s * v0; w[1] = s * v1; w[2] = s * v2;
+    w[0] = sc * v0; w[1] = sc * v1; w[2] = sc * v2;
   }
 }
 
-// inverse right Jacobian: I + 1/2 [w]x + c2 [w]x^2
+// c2 of the inverse right Jacobian I + 1/2 [w]x + c2 [w]x^2, t2 = |w|^2
+__device__ __forceinline__ double jr_inv_c2(double t2) {
+  if (t2 < kSmallAngle2) return 1.0 / 12.0 + t2 * (1.0 / 720.0 + t2 * (1.0 / 30240.0 + t2 * (1.0 / 1209600.0)));
+  const double t = sqrt(t2);
+  double s, c;
+  sincos(t, &s, &c);
+  return 1.0 / t2 - (1.0 + c) / (2.0 * t * s);
+}
 __device__ inline void so3_jr_inv(const double w[3], double J[9]) {
   const double t2 = w[0] * w[0] + w[1] * w[1] + w[2] * w[2];
-  double c2;
-  if (t2 < kSmallAngle2) {
-    c2 = 1.0 / 12.0 + t2 * (1.0 / 720.0 + t2 * (1.0 / 30240.0 + t2 * (1.0 / 1209600.0)));
-  } else {
-    const double t = sqrt(t2);
-    double s, c;
-    sincos(t, &s, &c);
-    c2 = 1.0 / t2 - (1.0 + c) / (2.0 * t * s);
-  }
+  const double c2 = jr_inv_c2(t2);
   const double d = 1.0 - c2 * t2;
   J[0] = d + c2 * w[0] * w[0];
   J[4] = d + c2 * w[1] * w[1];
@@ -212,6 +215,66 @@ __device__ inline double prior_terms(const double* R, const double* T, const dou
     }
   }
   return cost;
+}
+
+// The priors four lanes per image (a binary64 instruction occupies its quarter
+// of the SM for 64 cycles per warp, however many lanes take part, so what
+// counts is the length of a lane's program): lane q of the four takes axis q,
+// q = 0 .. 2 (the fourth lane repeats axis 2).  mask: the four lanes.
+__device__ __forceinline__ double quad_get(unsigned mask, double v, int q) {
+  return __shfl_sync(mask, v, ((threadIdx.x & 31) & ~3) | q);
+}
+// w: the rotation vector of Rp^T R
+__device__ __forceinline__ void quad_log(unsigned mask, const double* Rp, const double* R, int q, double w[3]) {
+  // E(i, j) = sum_k Rp(k, i) R(k, j); this lane: E(q, q) and the axial part
+  // E(a, b) - E(b, a), (a, b) = (2, 1), (0, 2), (1, 0)
+  const int a = q == 0 ? 2 : (q == 1 ? 0 : 1), b = q == 0 ? 1 : (q == 1 ? 2 : 0);
+  double tr = 0.0, v = 0.0, u = 0.0;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    tr += Rp[3 * k + q] * R[3 * k + q];
+    v += Rp[3 * k + a] * R[3 * k + b];
+    u += Rp[3 * k + b] * R[3 * k + a];
+  }
+  const double t0 = quad_get(mask, tr, 0), t1 = quad_get(mask, tr, 1), t2 = quad_get(mask, tr, 2);
+  const double s = log_scale(t0 + t1 + t2);
+  if (s >= 0.0) {
+    const double wq = s * (v - u);
+    for (int i = 0; i < 3; ++i) w[i] = quad_get(mask, wq, i);
+  } else {  // near a half turn: the general function
+    double E[9];
+    for (int i = 0; i < 3; ++i)
+      for (int j = 0; j < 3; ++j) E[3 * i + j] = Rp[i] * R[j] + Rp[3 + i] * R[3 + j] + Rp[6 + i] * R[6 + j];
+    so3_log(E, w);
+  }
+}
+
+// Prior cost of image k at (R, T), all four lanes
+static __device__ __noinline__ double prior_cost_quad(unsigned mask, const DevCluster& C, int k, const double* R,
+                                               const double* T, int q) {
+  double v = 0.0;
+  if (C.inv_imu2 > 0.0) {
+    double w[3];
+    quad_log(mask, C.R_prior + 9 * k, R, q, w);
+    v = 0.5 * C.inv_imu2 * (w[0] * w[0] + w[1] * w[1] + w[2] * w[2]);
+  }
+  if (C.inv_gnss2 > 0.0) {
+    const double e = T[q] - C.T_prior[3 * k + q];
+    double e2 = 0.0;
+    for (int i = 0; i < 3; ++i) {
+      const double ei = quad_get(mask, e, i);
+      e2 += ei * ei;
+    }
+    v += 0.5 * C.inv_gnss2 * e2;
+  }
+  return v;
+}
+
+// Sum of t[0 .. m) by one warp, in a fixed order; valid in lane 0
+__device__ __forceinline__ double strided_sum(const double* t, int m, int lane) {
+  double v = 0.0;
+  for (int j = lane; j < m; j += 32) v += t[j];
+  return warp_sum(v);
 }
 
 // ------------------------------------------------------------------ Eq. 5 + Brown, Eq. 6

@@ -117,6 +117,7 @@ struct DevCluster {
   int n_cams, n_pts, n_obs, n_free;
   int n_tiles, n_chunks, n_pairs, n_cslots, n_pslots, pad_i;
   double sigma_px, huber_delta, sigma_gnss, sigma_imu;
+  double inv_gnss2, inv_imu2;  // 1 / sigma^2 of the priors, 0 when off
   float inv_sigma_f, delta_f, half_inv_s2_f, pad_f;  // binary32 copies of 1/sigma_px, delta, 1/(2 sigma_px^2)
 
   const double* intr;      // [nc][7]
@@ -209,8 +210,7 @@ struct BatchView {
   // launch parameters the autotuner chooses (TuneParams)
   int lin_ctas_per_sm;   // linearise+Schur grid: at most this many CTAs per SM (grid-stride beyond)
   int back_ctas_per_sm;  // back-substitution grid: at most this many CTAs per SM
-  int factor_nb;         // panel width of the shared-memory Cholesky
-  int factor_threads;    // threads of the shared-memory factor CTA
+  int factor_threads;    // twice the threads of the shared-memory factor's CTAs (at least 192 each)
   int factor_df;         // 1: the shared-memory factor in double-float (mixed path, or BA_FLAG_SMALL_DF_FACTOR)
 };
 
@@ -219,7 +219,7 @@ struct TuneParams {
   int chunk_tiles = 0;       // tiles per linearise+Schur chunk (0: the precision's maximum)
   int lin_ctas_per_sm = 8;
   int back_ctas_per_sm = 16;
-  int factor_nb = 8;
+  int factor_nb = 8;         // kept for its place in the interface: the factor's block columns are 8 wide
   int factor_threads = 512;
   int big_panel_w = 4;       // columns of a block of the global-memory solver's panel factorisation
   int batch_chains = 4;      // concurrent launch chains of a batch's LM iterations
@@ -330,7 +330,11 @@ void launch_patch_poses(int n, const double* p0, const double* intr0, const doub
 // c, g0: host arrays of 2
 void launch_patch_planar(int n, const double* q0, const double* c, const double* g0, int m, const double* theta,
                          const double* g, double* q, cudaStream_t st);
+// the reduced systems of up to kMaxFreeSmall free images (ba_factor.cu);
+// assemble_only: g_c alone
 size_t factor_smem_bytes(int max_n);
+cudaError_t set_factor_attributes(int max_n);
+void launch_factor(const BatchView& bv, bool mixed, int refine_steps, int assemble_only, cudaStream_t st);
 void launch_fma_probe(int ctas, int iters, float* sink, cudaStream_t st);
 int chunk_obs(bool mixed);
 int chunk_tiles(bool mixed);

@@ -932,10 +932,14 @@ __device__ __forceinline__ typename AccOf<Real>::T add_rows(const Real* part, in
 struct RedItem {
   const int* slots;
   const void* part;
-  double* out;
   int begin, n, width;  // n = 0: nothing to do (its cluster is inactive, or no such item)
+  // element e of the sums: out[(e / 6) si + (e % 6) sc], negated for a pair
+  // block of a cluster of up to kMaxFreeSmall free images, which goes to its
+  // place in S (elimination order, lower triangle; and mirrored to out2)
+  double *out, *out2;
+  int si, sc;
 };
-__device__ __forceinline__ RedItem red_item(const BatchView& bv, int g) {
+__device__ __forceinline__ RedItem red_item(const BatchView& bv, int g, int mirror) {
   const int s = find_slot(bv.item_pre, bv.n, g);
   const DevCluster& C = bv.cl[s];
   if (!C.lm->active) return RedItem{};
@@ -948,13 +952,37 @@ __device__ __forceinline__ RedItem red_item(const BatchView& bv, int g) {
   r.n = begin[1] - r.begin;
   r.slots = cam ? C.cam_slots : C.pair_slots;
   r.part = cam ? C.campart : C.pairpart;
-  r.out = cam ? C.camsum + (size_t)kCamPart * key : C.pairsum + (size_t)kPairPart * key;
+  r.out2 = nullptr;
+  r.si = 6;
+  r.sc = 1;
   r.width = cam ? 39 : 36;
+  if (cam) {
+    r.out = C.camsum + (size_t)kCamPart * key;
+  } else if (C.n_free > kMaxFreeSmall) {
+    r.out = C.pairsum + (size_t)kPairPart * key;
+  } else {  // -(sum Z_a Z_b^T): rows a, columns b, or its transpose below the diagonal
+    const int n = 6 * C.n_free;
+    const int2 ab = C.pair_key[key];
+    const int pa = 6 * C.fpos[ab.x], pb = 6 * C.fpos[ab.y];
+    double* const rows_a = C.S + (size_t)pa * n + pb;
+    double* const rows_b = C.S + (size_t)pb * n + pa;
+    r.out = pa > pb ? rows_a : rows_b;
+    r.si = pa > pb ? n : 1;
+    r.sc = pa > pb ? 1 : n;
+    if (mirror) r.out2 = pa > pb ? rows_b : rows_a;
+    r.width = -36;
+  }
   return r;
+}
+__device__ __forceinline__ void red_store(const RedItem& r, int el, double v) {
+  const int i = el / 6, c = el - 6 * i;
+  if (r.width < 0) v = -v;
+  r.out[(size_t)i * r.si + (size_t)c * r.sc] = v;
+  if (r.out2) r.out2[(size_t)i * r.sc + (size_t)c * r.si] = v;
 }
 
 template <typename Real>
-__global__ void __launch_bounds__(kRedThreads) k_partial_reduce(BatchView bv) {
+__global__ void __launch_bounds__(kRedThreads, 5) k_partial_reduce(BatchView bv, int mirror) {
   using Acc = typename AccOf<Real>::T;
   __shared__ typename Acc::Raw sums[2][kRedSegs][kCamPart];  // two items' worth: one barrier per long item
   __shared__ RedItem items[kRedSegs];
@@ -967,25 +995,25 @@ __global__ void __launch_bounds__(kRedThreads) k_partial_reduce(BatchView bv) {
     if (threadIdx.x < group) {
       const int g = g0 + threadIdx.x * gridDim.x;
       RedItem r{};
-      if (g < total) r = red_item(bv, g);
+      if (g < total) r = red_item(bv, g, mirror);
       items[threadIdx.x] = r;
     }
     __syncthreads();
     if (seg < group) {  // the short lists, a group each
       const RedItem r = items[seg];
-      if (r.n > 0 && r.n <= kRedLong && el < r.width) {
+      if (r.n > 0 && r.n <= kRedLong && el < abs(r.width)) {
         const Real* part = (const Real*)r.part + el;
-        const int stride = r.width == 36 ? kPairPart : kCamPart;
-        r.out[el] = add_rows<Real>(part, stride, r.slots, r.begin, r.begin + r.n).get();
+        const int stride = abs(r.width) == 36 ? kPairPart : kCamPart;
+        red_store(r, el, add_rows<Real>(part, stride, r.slots, r.begin, r.begin + r.n).get());
       }
     }
     for (int i = 0; i < group; ++i) {  // the long ones, all groups together
       const RedItem r = items[i];
       if (r.n <= kRedLong) continue;
-      const bool live = seg < kRedSegs && el < r.width;
+      const bool live = seg < kRedSegs && el < abs(r.width);
       if (live) {
         const Real* part = (const Real*)r.part + el;
-        const int stride = r.width == 36 ? kPairPart : kCamPart;
+        const int stride = abs(r.width) == 36 ? kPairPart : kCamPart;
         const int per = (r.n + kRedSegs - 1) / kRedSegs;
         const int p0 = r.begin + seg * per, p1 = r.begin + min(r.n, (seg + 1) * per);
         sums[buf][seg][el] = add_rows<Real>(part, stride, r.slots, p0, p1).v;
@@ -995,773 +1023,11 @@ __global__ void __launch_bounds__(kRedThreads) k_partial_reduce(BatchView bv) {
         Acc t{sums[buf][0][el]};
 #pragma unroll
         for (int q = 1; q < kRedSegs; ++q) t = acc_join(t, Acc{sums[buf][q][el]});
-        r.out[el] = t.get();
+        red_store(r, el, t.get());
       }
       buf ^= 1;
     }
     __syncthreads();  // items[] is read no more
-  }
-}
-
-// ------------------------------------------------------------------ K4 (FP64)
-
-__device__ __forceinline__ int pk(int i, int j) { return (i * (i + 1)) / 2 + j; }  // packed lower, j <= i
-
-size_t factor_smem_bytes(int max_n) {
-  // packed A, per-camera sums and priors, x, b, t, inv_diag, the envelope and
-  // scale exponents (ints), the double-float solves' block inverses
-  const int nf = max_n / 6;
-  const size_t doubles = (size_t)max_n * (max_n + 1) / 2 + (size_t)nf * 40 + (size_t)nf * 42 + 5 * (size_t)max_n +
-                         (size_t)((max_n + 31) / 32) * (32 * 33 / 2) + 64;
-  return doubles * sizeof(double);
-}
-
-#ifndef BA_FACTOR_THREADS
-#define BA_FACTOR_THREADS 512
-#endif
-constexpr int kFactorThreads = BA_FACTOR_THREADS;  // threads of the shared-memory factor CTA
-
-constexpr int kSolveNB = 32;   // diagonal block of the triangular solves (one warp)
-
-// Blocked right-looking Cholesky A = L L^T of the packed lower matrix in
-// shared memory, by the whole CTA.  Per column j of a panel of nb
-// columns: warp 0 takes the pivot (square root and its reciprocal, once) and
-// the scaled entries of the panel's own rows; then every thread scales its
-// rows of column j and updates the panel's remaining columns.  After the
-// panel the trailing matrix is updated with it in 4x4 register tiles.
-// inv_diag[j] = 1 / L(j, j) is kept for the solves; colbuf: shared [n].
-// efirst[i]: first column of row i inside the envelope of A.  The factor has
-// no fill outside the envelope, so every product with an entry left of it
-// is zero and is skipped (the sums are unchanged).
-// Sets *fail (shared) when a pivot is not positive.
-__device__ void chol_blocked(double* A, int n, double* inv_diag, double* colbuf, const int* efirst, int* fail,
-                             int nb) {
-  const int tid = threadIdx.x, bs = blockDim.x;
-  for (int k0 = 0; k0 < n; k0 += nb) {
-    const int k1 = min(k0 + nb, n);
-    for (int j = k0; j < k1; ++j) {
-      if (tid < 32) {
-        const int lane = tid;
-        double inv = 0.0;
-        if (lane == 0) {
-          const double d = A[pk(j, j)];
-          if (!(d > 0.0)) *fail = 1;
-          inv = pivot_rsqrt(d > 0.0 ? d : 1.0);  // one reciprocal square root per pivot
-          const double r = (d > 0.0 ? d : 1.0) * inv;
-          A[pk(j, j)] = r;
-          inv_diag[j] = inv;
-        }
-        inv = __shfl_sync(BA_FULL_MASK, inv, 0);
-        if (j + 1 + lane < k1) colbuf[j + 1 + lane] = A[pk(j + 1 + lane, j)] * inv;
-      }
-      __syncthreads();
-      const double inv = inv_diag[j];
-      for (int i = j + 1 + tid; i < n; i += bs) {
-        if (efirst[i] > j) continue;  // L(i, j) = 0
-        const double l = A[pk(i, j)] * inv;
-        A[pk(i, j)] = l;
-        const int cmax = min(i, k1 - 1);
-        for (int c = j + 1; c <= cmax; ++c) A[pk(i, c)] -= l * colbuf[c];
-      }
-      __syncthreads();
-    }
-    if (*fail) return;
-    const int m = n - k1;  // trailing matrix rows/cols k1..n-1
-    if (m > 0) {
-      const int nt = (m + 3) >> 2;
-      const int ntiles = nt * (nt + 1) / 2;
-      for (int t = tid; t < ntiles; t += bs) {
-        int bi = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
-        while ((bi + 1) * (bi + 2) / 2 <= t) ++bi;
-        while (bi * (bi + 1) / 2 > t) --bi;
-        const int bc = t - bi * (bi + 1) / 2;
-        const int i0 = k1 + 4 * bi, c0 = k1 + 4 * bc;
-        // columns of the panel that can be nonzero in both row groups
-        int fi = n, fc = n;
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-          if (i0 + a < n) fi = min(fi, efirst[i0 + a]);
-          if (c0 + a < n) fc = min(fc, efirst[c0 + a]);
-        }
-        const int qlo = max(k0, max(fi, fc));
-        if (qlo >= k1) continue;
-        double acc[4][4];
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-          for (int b = 0; b < 4; ++b) acc[a][b] = 0.0;
-        for (int q = qlo; q < k1; ++q) {
-          double li[4], lc[4];
-#pragma unroll
-          for (int a = 0; a < 4; ++a) {
-            li[a] = i0 + a < n ? A[pk(i0 + a, q)] : 0.0;
-            lc[a] = c0 + a < n ? A[pk(c0 + a, q)] : 0.0;
-          }
-#pragma unroll
-          for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int b = 0; b < 4; ++b) acc[a][b] += li[a] * lc[b];
-        }
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-          for (int b = 0; b < 4; ++b) {
-            const int i = i0 + a, c = c0 + b;
-            if (i < n && c <= i) A[pk(i, c)] -= acc[a][b];
-          }
-      }
-      __syncthreads();
-    }
-  }
-}
-
-// Cholesky with one panel of look-ahead.  Warps 0-3 (group P) factor the
-// next panel while warps 4.. (group T) update the rest of the trailing matrix
-// with the current panel, so that the panel's sequential pivot chain runs
-// behind the trailing update.  Per panel p (columns [k0, k1), already
-// factored) and next panel [k1, k2): group P first updates the next panel's
-// columns with panel p, then factors them column by column, synchronising on
-// a named barrier of its 128 threads; group T updates columns >= k2.  The
-// writes of the two groups are disjoint and both only read panel p.  Same
-// envelope skipping as chol_blocked.  Requires blockDim.x > 128.
-__device__ __forceinline__ void bar_group_p() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
-
-// factor columns [k1, k2) (already updated by every earlier panel), group P only
-__device__ void chol_panel_p(double* A, int n, int k1, int k2, double* inv_diag, double* colbuf, const int* efirst,
-                             int* fail) {
-  const int tid = threadIdx.x;
-  for (int j = k1; j < k2; ++j) {
-    if (tid < 32) {
-      double inv = 0.0;
-      if (tid == 0) {
-        const double d = A[pk(j, j)];
-        if (!(d > 0.0)) *fail = 1;
-        inv = pivot_rsqrt(d > 0.0 ? d : 1.0);
-        A[pk(j, j)] = (d > 0.0 ? d : 1.0) * inv;
-        inv_diag[j] = inv;
-      }
-      inv = __shfl_sync(BA_FULL_MASK, inv, 0);
-      if (j + 1 + tid < k2) colbuf[j + 1 + tid] = A[pk(j + 1 + tid, j)] * inv;
-    }
-    bar_group_p();
-    const double inv = inv_diag[j];
-    for (int i = j + 1 + tid; i < n; i += 128) {
-      if (efirst[i] > j) continue;  // L(i, j) = 0
-      const double l = A[pk(i, j)] * inv;
-      A[pk(i, j)] = l;
-      const int cmax = min(i, k2 - 1);
-      for (int c = j + 1; c <= cmax; ++c) A[pk(i, c)] -= l * colbuf[c];
-    }
-    bar_group_p();
-  }
-}
-
-__device__ void chol_lookahead(double* A, int n, double* inv_diag, double* colbuf, const int* efirst, int* fail,
-                               int nb) {
-  const int tid = threadIdx.x;
-  const bool gp = tid < 128;
-  if (gp) chol_panel_p(A, n, 0, min(nb, n), inv_diag, colbuf, efirst, fail);
-  __syncthreads();
-  for (int k0 = 0; k0 < n; k0 += nb) {
-    if (*fail) return;
-    const int k1 = min(k0 + nb, n), k2 = min(k1 + nb, n);
-    if (gp) {
-      if (k1 < n) {
-        // the next panel's columns c in [k1, k2), rows i >= c, with panel p
-        const int w = k2 - k1;
-        for (int u = tid; u < (n - k1) * w; u += 128) {
-          const int i = k1 + u / w, c = k1 + u % w;
-          if (c > i) continue;
-          const int qlo = max(k0, max(efirst[i], efirst[c]));
-          double s = 0.0;
-          for (int q = qlo; q < k1; ++q) s += A[pk(i, q)] * A[pk(c, q)];
-          A[pk(i, c)] -= s;
-        }
-        bar_group_p();
-        chol_panel_p(A, n, k1, k2, inv_diag, colbuf, efirst, fail);
-      }
-    } else if (k2 < n) {
-      // trailing columns >= k2 with panel p, by the other warps
-      const int tt = tid - 128, nt_thr = blockDim.x - 128;
-      const int m = n - k2;
-      const int nt = (m + 3) >> 2;
-      const int ntiles = nt * (nt + 1) / 2;
-      for (int t = tt; t < ntiles; t += nt_thr) {
-        int bi = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
-        while ((bi + 1) * (bi + 2) / 2 <= t) ++bi;
-        while (bi * (bi + 1) / 2 > t) --bi;
-        const int bc = t - bi * (bi + 1) / 2;
-        const int i0 = k2 + 4 * bi, c0 = k2 + 4 * bc;
-        int fi = n, fc = n;
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-          if (i0 + a < n) fi = min(fi, efirst[i0 + a]);
-          if (c0 + a < n) fc = min(fc, efirst[c0 + a]);
-        }
-        const int qlo = max(k0, max(fi, fc));
-        if (qlo >= k1) continue;
-        double acc[4][4];
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-          for (int b = 0; b < 4; ++b) acc[a][b] = 0.0;
-        for (int q = qlo; q < k1; ++q) {
-          double li[4], lc[4];
-#pragma unroll
-          for (int a = 0; a < 4; ++a) {
-            li[a] = i0 + a < n ? A[pk(i0 + a, q)] : 0.0;
-            lc[a] = c0 + a < n ? A[pk(c0 + a, q)] : 0.0;
-          }
-#pragma unroll
-          for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int b = 0; b < 4; ++b) acc[a][b] += li[a] * lc[b];
-        }
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-          for (int b = 0; b < 4; ++b) {
-            const int i = i0 + a, c = c0 + b;
-            if (i < n && c <= i) A[pk(i, c)] -= acc[a][b];
-          }
-      }
-    }
-    __syncthreads();
-  }
-}
-
-// After the factorisation: L = Lu D with D = diag(L) and Lu unit lower
-// triangular; the strictly lower part of A is scaled to Lu in place (the
-// diagonal keeps L(j, j)), so that S = Lu D^2 Lu^T and the sweeps need no
-// division.
-__device__ void chol_unit_scale(double* A, const double* inv_diag, const int* efirst, int n) {
-  const int total = n * (n + 1) / 2;
-  for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
-    int i = (int)((sqrtf(8.0f * (float)idx + 1.0f) - 1.0f) * 0.5f);  // row of packed entry idx
-    while ((i + 1) * (i + 2) / 2 <= idx) ++i;
-    while (i * (i + 1) / 2 > idx) --i;
-    const int j = idx - i * (i + 1) / 2;
-    if (j < i && j >= efirst[i]) A[idx] *= inv_diag[j];
-  }
-}
-
-// Solve S x = b in place (b in shared memory) with S = Lu D^2 Lu^T, by the
-// whole CTA.  Per diagonal block of kSolveNB rows, warp 0 sweeps the unit
-// triangle (lane = row of the block); then one thread per row updates the
-// rest of the vector with the block's columns.  Entries left of a row's
-// envelope are zero and skipped.
-__device__ void chol_solve_blocked(const double* A, const double* inv_diag, const int* efirst, double* b, int n) {
-  const int tid = threadIdx.x, bs = blockDim.x, lane = tid & 31, wid = tid >> 5;
-  for (int k0 = 0; k0 < n; k0 += kSolveNB) {  // Lu z = b
-    const int k1 = min(k0 + kSolveNB, n);
-    if (wid == 0) {
-      const int i = k0 + lane;
-      double v = i < k1 ? b[i] : 0.0;
-      for (int j = k0; j < k1 - 1; ++j) {
-        const double z = __shfl_sync(BA_FULL_MASK, v, j - k0);
-        if (i > j && i < k1 && efirst[i] <= j) v -= A[pk(i, j)] * z;
-      }
-      if (i < k1) b[i] = v;
-    }
-    __syncthreads();
-    for (int i = k1 + tid; i < n; i += bs) {  // b_i -= sum_{q in block} Lu(i, q) z_q
-      const int q0 = max(k0, efirst[i]);
-      double s = 0.0;
-      for (int q = q0; q < k1; ++q) s += A[pk(i, q)] * b[q];
-      b[i] -= s;
-    }
-    __syncthreads();
-  }
-  // w = D^-2 z, one factor 1 / L(i, i) at a time: the square of the
-  // reciprocal of a tiny (even subnormal) pivot would overflow
-  for (int i = tid; i < n; i += bs) b[i] = (b[i] * inv_diag[i]) * inv_diag[i];
-  __syncthreads();
-  const int nb = (n + kSolveNB - 1) / kSolveNB;
-  for (int blk = nb - 1; blk >= 0; --blk) {  // Lu^T x = w
-    const int k0 = blk * kSolveNB, k1 = min(k0 + kSolveNB, n);
-    if (wid == 0) {
-      const int i = k0 + lane;
-      double v = i < k1 ? b[i] : 0.0;
-      for (int j = k1 - 1; j > k0; --j) {
-        const double xj = __shfl_sync(BA_FULL_MASK, v, j - k0);
-        if (i < j && i >= k0 && efirst[j] <= i) v -= A[pk(j, i)] * xj;
-      }
-      if (i < k1) b[i] = v;
-    }
-    __syncthreads();
-    int lo = k0;  // the block's rows have no entry left of their envelopes
-    for (int q = k0; q < k1; ++q) lo = min(lo, efirst[q]);
-    for (int i = lo + tid; i < k0; i += bs) {  // b_i -= sum_{q in block} Lu(q, i) x_q
-      double s = 0.0;
-      for (int q = k0; q < k1; ++q)
-        if (efirst[q] <= i) s += A[pk(q, i)] * b[q];
-      b[i] -= s;
-    }
-    __syncthreads();
-  }
-}
-
-// ---- the same factorisation and solves in double-float (mixed path)
-//
-// The binary64 pipe of GB300 runs at 1/59 of the binary32 rate, and it bounds
-// the binary64 factor of the largest clusters (about 2 DFMA per clock per
-// SM).  The mixed path therefore factors an equilibrated copy of the system
-// in double-float on the binary32 pipe: A' = E A E with E = diag(2^e_i)
-// (powers of two, exact), e_i chosen so that A'(i, i) lies in [1/2, 4); the
-// diagonal near 1 keeps every entry of the factor well inside the binary32
-// exponent range whatever the scale of A.  A x = b is solved as A' y = E b,
-// x = E y; the iterative refinement against the binary64 S (unchanged)
-// removes the factor's rounding (double-float, about 2^-47 relative per
-// operation).  Same blocking, look-ahead and envelope skipping as the binary64
-// functions above; a pivot that is not positive sets *fail.
-
-// A (binary64, packed lower, envelope entries) -> A' = E A E as double-float
-// in the same bytes; escale[i] = e_i.  Entries left of a row's envelope are
-// zero in both representations.
-__device__ void chol_to_scaled_df(double* A, int n, const int* efirst, int* escale) {
-  const int tid = threadIdx.x, bs = blockDim.x, lane = tid & 31, wid = tid >> 5, nw = bs >> 5;
-  for (int i = tid; i < n; i += bs) {
-    const double d = A[pk(i, i)];
-    escale[i] = (d > 0.0 && d < INFINITY) ? -(ilogb(d) / 2) : 0;
-  }
-  __syncthreads();
-  dfl* Af = reinterpret_cast<dfl*>(A);
-  for (int i = wid; i < n; i += nw) {
-    const int ei = escale[i];
-    for (int j = efirst[i] + lane; j <= i; j += 32) Af[pk(i, j)] = df_from_d_pow2(A[pk(i, j)], ei + escale[j]);
-  }
-  __syncthreads();
-}
-
-__device__ __forceinline__ dfl shfl_df(dfl v, int src) {
-  return dfl{__shfl_sync(BA_FULL_MASK, v.hi, src), __shfl_sync(BA_FULL_MASK, v.lo, src)};
-}
-
-// factor columns [k1, k2) (already updated by every earlier panel), group P only
-__device__ void chol_panel_p_df(dfl* A, int n, int k1, int k2, dfl* inv_diag, dfl* colbuf, const int* efirst,
-                                int* fail) {
-  const int tid = threadIdx.x;
-  for (int j = k1; j < k2; ++j) {
-    if (tid < 32) {
-      dfl inv{0.0f, 0.0f};
-      if (tid == 0) {
-        dfl d = A[pk(j, j)];
-        if (!(d.hi > 0.0f)) {
-          *fail = 1;
-          d = dfl{1.0f, 0.0f};
-        }
-        inv = df_rsqrt(d);
-        A[pk(j, j)] = df_mul(d, inv);
-        inv_diag[j] = inv;
-      }
-      inv = shfl_df(inv, 0);
-      if (j + 1 + tid < k2) colbuf[j + 1 + tid] = df_mul(A[pk(j + 1 + tid, j)], inv);
-    }
-    bar_group_p();
-    const dfl inv = inv_diag[j];
-    for (int i = j + 1 + tid; i < n; i += 128) {
-      if (efirst[i] > j) continue;  // L(i, j) = 0
-      const dfl l = df_mul(A[pk(i, j)], inv);
-      A[pk(i, j)] = l;
-      const int cmax = min(i, k2 - 1);
-      for (int c = j + 1; c <= cmax; ++c) A[pk(i, c)] = df_fms(A[pk(i, c)], l, colbuf[c]);
-    }
-    bar_group_p();
-  }
-}
-
-__device__ void chol_lookahead_df(dfl* A, int n, dfl* inv_diag, dfl* colbuf, const int* efirst, int* fail, int nb) {
-  const int tid = threadIdx.x;
-  const bool gp = tid < 128;
-  if (gp) chol_panel_p_df(A, n, 0, min(nb, n), inv_diag, colbuf, efirst, fail);
-  __syncthreads();
-  for (int k0 = 0; k0 < n; k0 += nb) {
-    if (*fail) return;
-    const int k1 = min(k0 + nb, n), k2 = min(k1 + nb, n);
-    if (gp) {
-      if (k1 < n) {
-        const int w = k2 - k1;
-        for (int u = tid; u < (n - k1) * w; u += 128) {
-          const int i = k1 + u / w, c = k1 + u % w;
-          if (c > i) continue;
-          const int qlo = max(k0, max(efirst[i], efirst[c]));
-          if (qlo >= k1) continue;
-          Dot2 s;
-          for (int q = qlo; q < k1; ++q) s.add(A[pk(i, q)], A[pk(c, q)]);
-          A[pk(i, c)] = df_sub(A[pk(i, c)], s.get());
-        }
-        bar_group_p();
-        chol_panel_p_df(A, n, k1, k2, inv_diag, colbuf, efirst, fail);
-      }
-    } else if (k2 < n) {
-      const int tt = tid - 128, nt_thr = blockDim.x - 128;
-      const int m = n - k2;
-      const int nt = (m + 3) >> 2;
-      const int ntiles = nt * (nt + 1) / 2;
-      for (int t = tt; t < ntiles; t += nt_thr) {
-        int bi = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
-        while ((bi + 1) * (bi + 2) / 2 <= t) ++bi;
-        while (bi * (bi + 1) / 2 > t) --bi;
-        const int bc = t - bi * (bi + 1) / 2;
-        const int i0 = k2 + 4 * bi, c0 = k2 + 4 * bc;
-        int fi = n, fc = n;
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-          if (i0 + a < n) fi = min(fi, efirst[i0 + a]);
-          if (c0 + a < n) fc = min(fc, efirst[c0 + a]);
-        }
-        const int qlo = max(k0, max(fi, fc));
-        if (qlo >= k1) continue;
-        Dot2 acc[4][4];
-        for (int q = qlo; q < k1; ++q) {
-          dfl li[4], lc[4];
-#pragma unroll
-          for (int a = 0; a < 4; ++a) {
-            li[a] = i0 + a < n ? A[pk(i0 + a, q)] : dfl{0.0f, 0.0f};
-            lc[a] = c0 + a < n ? A[pk(c0 + a, q)] : dfl{0.0f, 0.0f};
-          }
-#pragma unroll
-          for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int b = 0; b < 4; ++b) acc[a][b].add(li[a], lc[b]);
-        }
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-          for (int b = 0; b < 4; ++b) {
-            const int i = i0 + a, c = c0 + b;
-            if (i < n && c <= i) A[pk(i, c)] = df_sub(A[pk(i, c)], acc[a][b].get());
-          }
-      }
-    }
-    __syncthreads();
-  }
-}
-
-__device__ void chol_unit_scale_df(dfl* A, const dfl* inv_diag, const int* efirst, int n) {
-  const int tid = threadIdx.x, bs = blockDim.x, lane = tid & 31, wid = tid >> 5, nw = bs >> 5;
-  (void)bs;
-  for (int i = wid; i < n; i += nw)
-    for (int j = efirst[i] + lane; j < i; j += 32) A[pk(i, j)] = df_mul(A[pk(i, j)], inv_diag[j]);
-}
-
-// Inverses of the unit-lower diagonal blocks of kSolveNB rows of Lu, packed
-// lower (entry (r, c) of a block at r (r + 1) / 2 + c, the unit diagonal
-// stored), one warp per block, lane = column c:
-// X(c, c) = 1, X(r, c) = -sum_{q=c}^{r-1} Lu(r, q) X(q, c) for r > c.
-// The solves then apply each block as a product instead of a sequential
-// substitution.
-constexpr int kSolveTri = kSolveNB * (kSolveNB + 1) / 2;
-__device__ void chol_block_inverses_df(const dfl* A, const int* efirst, dfl* binv, int n) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const int nb = (n + kSolveNB - 1) / kSolveNB;
-  for (int blk = wid; blk < nb; blk += nw) {
-    const int k0 = blk * kSolveNB, m = min(kSolveNB, n - k0);
-    dfl* X = binv + (size_t)blk * kSolveTri;
-    const int c = lane;
-    if (c >= m) continue;
-    X[c * (c + 1) / 2 + c] = dfl{1.0f, 0.0f};
-    for (int r = c + 1; r < m; ++r) {
-      const int qs = max(c, efirst[k0 + r] - k0);  // Lu(r, q) = 0 left of the envelope
-      const dfl* Lr = A + pk(k0 + r, k0);
-      Dot2 s0, s1;
-      int q = qs;
-      for (; q + 1 < r; q += 2) {
-        s0.add(Lr[q], X[q * (q + 1) / 2 + c]);
-        s1.add(Lr[q + 1], X[(q + 1) * (q + 2) / 2 + c]);
-      }
-      for (; q < r; ++q) s0.add(Lr[q], X[q * (q + 1) / 2 + c]);
-      s0.merge(s1.s, s1.c);
-      X[r * (r + 1) / 2 + c] = df_neg(s0.get());
-    }
-  }
-}
-
-// S' y = b in place with S' = Lu D^2 Lu^T (double-float): the sweeps of
-// chol_solve_blocked, each diagonal block applied through its inverse (warp
-// 0, lane = row), the rest of the vector updated thread per row, all sums
-// compensated (Dot2)
-__device__ void chol_solve_df(const dfl* A, const dfl* inv_diag, const int* efirst, const dfl* binv, dfl* b, int n) {
-  const int tid = threadIdx.x, bs = blockDim.x, lane = tid & 31, wid = tid >> 5;
-  for (int k0 = 0; k0 < n; k0 += kSolveNB) {  // Lu z = b
-    const int k1 = min(k0 + kSolveNB, n);
-    if (wid == 0) {
-      const dfl* X = binv + (size_t)(k0 / kSolveNB) * kSolveTri;
-      const int r = lane, i = k0 + r;
-      dfl v{0.0f, 0.0f};
-      if (i < k1) {  // z_r = sum_{q <= r} X(r, q) b_q
-        const dfl* Xr = X + r * (r + 1) / 2;
-        Dot2 s0, s1;
-        int q = 0;
-        for (; q + 1 <= r; q += 2) {
-          s0.add(Xr[q], b[k0 + q]);
-          s1.add(Xr[q + 1], b[k0 + q + 1]);
-        }
-        for (; q <= r; ++q) s0.add(Xr[q], b[k0 + q]);
-        s0.merge(s1.s, s1.c);
-        v = s0.get();
-      }
-      __syncwarp();
-      if (i < k1) b[i] = v;
-    }
-    __syncthreads();
-    for (int i = k1 + tid; i < n; i += bs) {
-      const int q0 = max(k0, efirst[i]);
-      if (q0 >= k1) continue;
-      Dot2 s0, s1, s2, s3;  // four interleaved sums, merged in a fixed order
-      int q = q0;
-      for (; q + 3 < k1; q += 4) {
-        s0.add(A[pk(i, q)], b[q]);
-        s1.add(A[pk(i, q + 1)], b[q + 1]);
-        s2.add(A[pk(i, q + 2)], b[q + 2]);
-        s3.add(A[pk(i, q + 3)], b[q + 3]);
-      }
-      for (; q < k1; ++q) s0.add(A[pk(i, q)], b[q]);
-      s0.merge(s1.s, s1.c);
-      s2.merge(s3.s, s3.c);
-      s0.merge(s2.s, s2.c);
-      b[i] = df_sub(b[i], s0.get());
-    }
-    __syncthreads();
-  }
-  for (int i = tid; i < n; i += bs) b[i] = df_mul(df_mul(b[i], inv_diag[i]), inv_diag[i]);  // D^-2
-  __syncthreads();
-  const int nb = (n + kSolveNB - 1) / kSolveNB;
-  for (int blk = nb - 1; blk >= 0; --blk) {  // Lu^T x = w
-    const int k0 = blk * kSolveNB, k1 = min(k0 + kSolveNB, n), m = k1 - k0;
-    if (wid == 0) {
-      const dfl* X = binv + (size_t)blk * kSolveTri;
-      const int r = lane, i = k0 + r;
-      dfl v{0.0f, 0.0f};
-      if (i < k1) {  // x_r = sum_{q >= r} X(q, r) w_q
-        Dot2 s0, s1;
-        int q = r;
-        for (; q + 1 < m; q += 2) {
-          s0.add(X[q * (q + 1) / 2 + r], b[k0 + q]);
-          s1.add(X[(q + 1) * (q + 2) / 2 + r], b[k0 + q + 1]);
-        }
-        for (; q < m; ++q) s0.add(X[q * (q + 1) / 2 + r], b[k0 + q]);
-        s0.merge(s1.s, s1.c);
-        v = s0.get();
-      }
-      __syncwarp();
-      if (i < k1) b[i] = v;
-    }
-    __syncthreads();
-    int lo = k0;
-    for (int q = k0; q < k1; ++q) lo = min(lo, efirst[q]);
-    for (int i = lo + tid; i < k0; i += bs) {
-      // the block's rows whose envelope reaches column i are a prefix
-      // [k0, qe) of it (the envelope is monotone)
-      int qe = k0;
-      while (qe < k1 && efirst[qe] <= i) ++qe;
-      if (qe == k0) continue;
-      Dot2 s0, s1, s2, s3;
-      int q = k0;
-      for (; q + 3 < qe; q += 4) {
-        s0.add(A[pk(q, i)], b[q]);
-        s1.add(A[pk(q + 1, i)], b[q + 1]);
-        s2.add(A[pk(q + 2, i)], b[q + 2]);
-        s3.add(A[pk(q + 3, i)], b[q + 3]);
-      }
-      for (; q < qe; ++q) s0.add(A[pk(q, i)], b[q]);
-      s0.merge(s1.s, s1.c);
-      s2.merge(s3.s, s3.c);
-      s0.merge(s2.s, s2.c);
-      b[i] = df_sub(b[i], s0.get());
-    }
-    __syncthreads();
-  }
-}
-
-// A x = v for the binary64 vector v (in place): scaled into double-float in
-// the same bytes, solved, scaled back
-__device__ void solve_scaled_df(const dfl* A, const dfl* inv_diag, const int* efirst, const int* escale,
-                                const dfl* binv, double* v, int n) {
-  dfl* vf = reinterpret_cast<dfl*>(v);
-  for (int i = threadIdx.x; i < n; i += blockDim.x) vf[i] = df_from_d_pow2(v[i], escale[i]);
-  __syncthreads();
-  chol_solve_df(A, inv_diag, efirst, binv, vf, n);
-  for (int i = threadIdx.x; i < n; i += blockDim.x) v[i] = ldexp(df_to_d(vf[i]), escale[i]);
-  __syncthreads();
-}
-
-template <bool MIXED>
-__global__ void __launch_bounds__(kFactorThreads) k_factor_solve(BatchView bv, int refine_steps, int assemble_only) {
-  using Real = typename RealOf<MIXED>::T;
-  extern __shared__ double sm[];
-  __shared__ int fail;
-  const int tid = threadIdx.x, bs = blockDim.x;
-  for (int so = blockIdx.x; so < bv.n; so += gridDim.x) {
-    const int s = bv.factor_order[so];  // largest systems first
-    const DevCluster& C = bv.cl[s];
-    LmState* lm = C.lm;
-    if (!lm->active && !assemble_only) continue;
-    if (C.n_free > kMaxFreeSmall) continue;  // the global-memory solver takes larger systems
-    const int nf = C.n_free, n = 6 * nf, nc = C.n_cams;
-    const double mu = lm->mu;
-    const int cur = lm->cur;
-    double* A = sm;
-    double* cd = A + (size_t)n * (n + 1) / 2;  // [nf][40]
-    double* pr = cd + (size_t)nf * 40;         // [nf][42]: JtJ 36, Jtr 6
-    double* x = pr + (size_t)nf * 42;          // [n]
-    double* b = x + n;                         // [n]
-    double* t = b + n;                         // [n]
-    double* inv_diag = t + n;                  // [n]
-    const double* Rc = C.R + (size_t)cur * nc * 9;
-    const double* Tc = C.T + (size_t)cur * nc * 3;
-
-    if (tid == 0) lm->tiles_done = 0;  // the back-substitution counts its tiles from here
-    // per-camera sums (k_partial_reduce)
-    for (int idx = tid; idx < nf * 39; idx += bs) {
-      const int f = idx / 39, e = idx - 39 * f;
-      cd[40 * f + e] = C.camsum[(size_t)kCamPart * f + e];
-    }
-    for (int f = tid; f < nf; f += bs) {
-      const int k = C.cam_of_free[f];
-      prior_terms(Rc + 9 * k, Tc + 3 * k, C.R_prior + 9 * k, C.T_prior + 3 * k, C.sigma_imu, C.sigma_gnss,
-                  pr + 42 * f, pr + 42 * f + 36);
-    }
-    for (int idx = tid; idx < n * (n + 1) / 2; idx += bs) A[idx] = 0.0;
-    if (tid == 0) fail = lm->pt_fail;
-    __syncthreads();
-    // diagonal blocks: U + prior + mu D - sum Z Z^T
-    for (int idx = tid; idx < nf * 21; idx += bs) {
-      const int f = idx / 21;
-      int e = idx - 21 * f, a = 0;
-      while (e >= 6 - a) { e -= 6 - a; ++a; }
-      const int bb = a + e;  // a <= bb, packed upper index of (a, bb)
-      const int ui = idx - 21 * f;
-      double v = cd[40 * f + ui] + pr[42 * f + 6 * a + bb];
-      if (a == bb) {
-        const double D = clamp_diag(cd[40 * f + 33 + a] + pr[42 * f + 7 * a]);
-        v += mu * D;
-        C.Dc[6 * f + a] = D;
-      }
-      const int p = C.fpos[f];
-      A[pk(6 * p + bb, 6 * p + a)] = v;  // row bb >= col a
-    }
-    for (int idx = tid; idx < n; idx += bs) {
-      const int f = idx / 6, a = idx - 6 * f;
-      const double g = cd[40 * f + 21 + a] - pr[42 * f + 36 + a];
-      C.gc[idx] = g;
-      const double r = g - cd[40 * f + 27 + a];
-      const int pi = 6 * C.fpos[f] + a;  // elimination order
-      C.rhs[pi] = r;
-      b[pi] = r;
-    }
-    // off-diagonal blocks: S(fb, fa) = -(sum Z_a Z_b^T)^T
-    for (int idx = tid; idx < C.n_pairs * 36; idx += bs) {
-      const int p = idx / 36, e = idx - 36 * p;
-      const int i = e / 6, c = e - 6 * i;
-      const double v = C.pairsum[(size_t)kPairPart * p + e];
-      const int2 key = C.pair_key[p];
-      const int pa = C.fpos[key.x], pb = C.fpos[key.y];
-      if (pb > pa) A[pk(6 * pb + c, 6 * pa + i)] = -v;
-      else A[pk(6 * pa + i, 6 * pb + c)] = -v;
-    }
-    __syncthreads();
-    if (assemble_only || refine_steps > 0) {  // S in binary64 for the refinement (only the refinement reads it)
-      for (int idx = tid; idx < n * n; idx += bs) {
-        const int r = idx / n, c = idx - n * r;
-        C.S[idx] = r >= c ? A[pk(r, c)] : A[pk(c, r)];
-      }
-    }
-    if (assemble_only) {
-      __syncthreads();
-      continue;
-    }
-    __syncthreads();  // the copy of S above reads A
-    // blocked right-looking Cholesky in shared memory (t[] is the column buffer)
-    int* efirst = reinterpret_cast<int*>(inv_diag + n);  // [n]: first column of each row's envelope
-    for (int idx = tid; idx < n; idx += bs) efirst[idx] = 6 * C.env_first[idx / 6];
-    __syncthreads();
-    // double-float factor of the equilibrated system (escale: its exponents):
-    // the mixed path, and the binary64 path under BA_FLAG_SMALL_DF_FACTOR
-    const bool use_df = MIXED || bv.factor_df;
-    int* escale = efirst + n;
-    dfl* binv = reinterpret_cast<dfl*>(inv_diag + 2 * n);  // inverses of the solves' diagonal blocks
-    dfl* Af = reinterpret_cast<dfl*>(A);
-    dfl* inv_f = reinterpret_cast<dfl*>(inv_diag);
-    if (use_df) {
-      chol_to_scaled_df(A, n, efirst, escale);
-      if (!fail) chol_lookahead_df(Af, n, inv_f, reinterpret_cast<dfl*>(t), efirst, &fail, bv.factor_nb);
-    } else {
-#ifdef BA_FACTOR_NO_LOOKAHEAD
-      if (!fail) chol_blocked(A, n, inv_diag, t, efirst, &fail, bv.factor_nb);
-#else
-      if (!fail) chol_lookahead(A, n, inv_diag, t, efirst, &fail, bv.factor_nb);
-#endif
-    }
-    __syncthreads();
-    const int status = fail ? BA_STATUS_NOT_PD : 0;
-    if (!fail) {
-      if (use_df) {
-        chol_unit_scale_df(Af, inv_f, efirst, n);
-        __syncthreads();
-        chol_block_inverses_df(Af, efirst, binv, n);
-        __syncthreads();
-        solve_scaled_df(Af, inv_f, efirst, escale, binv, b, n);
-      } else {
-        chol_unit_scale(A, inv_diag, efirst, n);
-        __syncthreads();
-        chol_solve_blocked(A, inv_diag, efirst, b, n);
-      }
-      for (int idx = tid; idx < n; idx += bs) x[idx] = b[idx];
-      __syncthreads();
-      // iterative refinement against the FP64 system kept in global memory
-      for (int it = 0; it < refine_steps; ++it) {
-        const int lane = tid & 31, wid = tid >> 5, nw = bs >> 5;
-        for (int r = wid; r < n; r += nw) {
-          double acc = 0.0;
-          for (int c = efirst[r] + lane; c < n; c += 32)  // zero blocks outside the envelope skipped
-            if (c <= r || efirst[c] <= r) acc += C.S[(size_t)r * n + c] * x[c];
-          acc = warp_sum(acc);
-          if (lane == 0) t[r] = C.rhs[r] - acc;
-        }
-        __syncthreads();
-        if (use_df) solve_scaled_df(Af, inv_f, efirst, escale, binv, t, n);
-        else chol_solve_blocked(A, inv_diag, efirst, t, n);
-        for (int idx = tid; idx < n; idx += bs) x[idx] += t[idx];
-        __syncthreads();
-      }
-      for (int idx = tid; idx < n; idx += bs) {  // back to free-image order
-        const double v = x[6 * C.fpos[idx / 6] + idx % 6];
-        C.dc[idx] = v;
-        if (MIXED) C.dc32[idx] = (float)v;
-      }
-    } else {
-      for (int idx = tid; idx < n; idx += bs) {
-        C.dc[idx] = 0.0;
-        if (MIXED) C.dc32[idx] = 0.0f;
-        x[idx] = 0.0;
-      }
-    }
-    __syncthreads();
-    // candidate cameras; per-camera prior cost and pred terms into t[]
-    for (int k = tid; k < nc; k += bs) {
-      const int f = C.free_idx[k];
-      double pc, pn;
-      candidate_camera<MIXED>(C, k, x, mu, cur, fail != 0, &pc, &pn);
-      if (f >= 0) {
-        t[2 * f] = pc;
-        t[2 * f + 1] = pn;
-      }
-    }
-    __syncthreads();
-    if (tid == 0) {
-      double pc = 0.0, pn = 0.0;
-      for (int f = 0; f < nf; ++f) { pc += t[2 * f]; pn += t[2 * f + 1]; }
-      lm->pred_cam = pc;
-      lm->prior_new = pn;
-      lm->status = lm->dev_error ? lm->dev_error : status;
-      lm->dev_error = 0;
-    }
-    __syncthreads();
-    // a cluster without observations has no back-substitution tile to count:
-    // its LM step is taken here
-    if (!assemble_only && C.n_tiles == 0 && tid < 32) lm_update_warp<MIXED>(C, tid);
-    __syncthreads();
   }
 }
 
@@ -2065,22 +1331,35 @@ __device__ double block_sum(double v, double* red) {
 }
 
 __global__ void __launch_bounds__(256) k_cost_init(BatchView bv) {
-  __shared__ double red[8];
+  __shared__ double red[8], prior[kMaxFreeSmall];
   for (int s = blockIdx.x; s < bv.n; s += gridDim.x) {
     const DevCluster& C = bv.cl[s];
     LmState* lm = C.lm;
     if (!lm->needs_init) continue;
     const double F = block_sum_tiles(C, 0, red);
-    // prior terms of the free images at the current state: thread t takes
-    // images t, t + blockDim.x, ... in order
     const int cur = lm->cur;
+    const double* R = C.R + (size_t)cur * C.n_cams * 9;
+    const double* T = C.T + (size_t)cur * C.n_cams * 3;
     double pc = 0.0;
-    for (int k = threadIdx.x; k < C.n_cams; k += blockDim.x) {
-      if (C.free_idx[k] < 0) continue;
-      pc += prior_terms(C.R + ((size_t)cur * C.n_cams + k) * 9, C.T + ((size_t)cur * C.n_cams + k) * 3,
-                        C.R_prior + 9 * k, C.T_prior + 3 * k, C.sigma_imu, C.sigma_gnss, nullptr, nullptr);
+    if (C.n_free <= kMaxFreeSmall) {
+      // as the factor kernel forms it at a candidate, so that F carried from
+      // there and F evaluated here are the same bits
+      if (threadIdx.x < 4 * C.n_free) {
+        const int f = threadIdx.x >> 2, k = C.cam_of_free[f], q = min((int)threadIdx.x & 3, 2);
+        const double v = prior_cost_quad(0xfu << ((threadIdx.x & 31) & ~3), C, k, R + 9 * k, T + 3 * k, q);
+        if ((threadIdx.x & 3) == 0) prior[f] = v;
+      }
+      __syncthreads();
+      if (threadIdx.x < 32) pc = strided_sum(prior, C.n_free, threadIdx.x);
+    } else {
+      // thread t takes images t, t + blockDim.x, ... in order
+      for (int k = threadIdx.x; k < C.n_cams; k += blockDim.x) {
+        if (C.free_idx[k] < 0) continue;
+        pc += prior_terms(R + 9 * k, T + 3 * k, C.R_prior + 9 * k, C.T_prior + 3 * k, C.sigma_imu, C.sigma_gnss, nullptr,
+                          nullptr);
+      }
+      pc = block_sum(pc, red);
     }
-    pc = block_sum(pc, red);
     if (threadIdx.x == 0) {
       lm->needs_init = 0;
       lm->F = F + pc;
@@ -2449,19 +1728,17 @@ static void launch_lin_schur(const BatchView& bv, int diag, cudaStream_t st) {
 
 
 template <bool MIXED>
-static void launch_partial_reduce(const BatchView& bv, cudaStream_t st) {
+static void launch_partial_reduce(const BatchView& bv, int mirror, cudaStream_t st) {
   using Real = typename RealOf<MIXED>::T;
-  LAUNCH(KK_PARTIAL_REDUCE, st, k_partial_reduce<Real><<<grid_for(bv.total_items, 1, num_sms() * kRedCtasPerSm), kRedThreads, 0, st>>>(bv));
+  LAUNCH(KK_PARTIAL_REDUCE, st, k_partial_reduce<Real><<<grid_for(bv.total_items, 1, num_sms() * kRedCtasPerSm), kRedThreads, 0, st>>>(bv, mirror));
 }
 
 template <bool MIXED>
 static void launch_iteration_t(const BatchView& bv, int refine_steps, cudaStream_t st, const std::vector<BigRef>* big) {
   const int sms = num_sms();
   launch_lin_schur<MIXED>(bv, 0, st);
-  launch_partial_reduce<MIXED>(bv, st);
-  const size_t smem = factor_smem_bytes(bv.max_n);
-  LAUNCH(KK_FACTOR, st,
-         k_factor_solve<MIXED><<<grid_for(bv.n, 1, 65535), bv.factor_threads, smem, st>>>(bv, refine_steps, 0));
+  launch_partial_reduce<MIXED>(bv, refine_steps > 0, st);
+  launch_factor(bv, MIXED, refine_steps, 0, st);
   if (big)
     for (const BigRef& b : *big) launch_big_solve(b, MIXED, refine_steps, 0, st);
   LAUNCH(KK_BACKSUB, st, k_backsub_cost<MIXED><<<grid_for(bv.total_tiles, 8, sms * bv.back_ctas_per_sm), kCostInitThreads, 0, st>>>(bv));
@@ -2476,9 +1753,8 @@ void launch_iteration(const BatchView& bv, bool mixed, int refine_steps, cudaStr
 template <bool MIXED>
 static void launch_grad_norm_t(const BatchView& bv, double* out, cudaStream_t st, const std::vector<BigRef>* big) {
   launch_lin_schur<MIXED>(bv, 1, st);
-  launch_partial_reduce<MIXED>(bv, st);
-  LAUNCH(KK_FACTOR, st,
-         k_factor_solve<MIXED><<<grid_for(bv.n, 1, 65535), bv.factor_threads, factor_smem_bytes(bv.max_n), st>>>(bv, 0, 1));
+  launch_partial_reduce<MIXED>(bv, 0, st);
+  launch_factor(bv, MIXED, 0, 1, st);
   if (big)
     for (const BigRef& b : *big) launch_big_solve(b, MIXED, 0, 1, st);
   LAUNCH(KK_OTHER, st, k_grad_norm<<<grid_for(bv.n, 1, 65535), 256, 0, st>>>(bv, out));
@@ -2522,10 +1798,7 @@ void launch_fma_probe(int ctas, int iters, float* sink, cudaStream_t st) {
 }
 
 cudaError_t set_kernel_attributes(int max_n) {
-  const size_t smem = factor_smem_bytes(max_n);
-  cudaError_t e = cudaFuncSetAttribute(k_factor_solve<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_factor_solve<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = set_factor_attributes(max_n);
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_lin_schur<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)chunk_smem_bytes(true));
   if (e != cudaSuccess) return e;
