@@ -885,8 +885,10 @@ __device__ __forceinline__ AccD acc_join(AccD a, AccD b) { return AccD{a.v + b.v
 // chunk partials, added, into camsum / pairsum.
 //
 // Per iteration on GB300: one cluster of 235 k observations 39 -> 12 us (97 ->
-// 18 in binary64), 12 clusters 25 -> 17, 400 images 24 -> 27, 128 clusters
-// 68 -> 76 (their short lists filled the GPU as a warp each too).
+// 19 in binary64), 12 clusters 25 -> 21, 128 clusters 68 -> 83: their short
+// lists filled the GPU as a warp each too, and the pair sums go to their rows
+// in S here (a wider spread of stores, 98 us when the transposed ones went out
+// column by column), which saves the factor its pair tables.
 //
 // What bounds it is the latency of the loads: an item is a list of rows, up
 // to one per chunk of the cluster (501 of them for 235 k observations), and
@@ -902,7 +904,7 @@ __device__ __forceinline__ AccD acc_join(AccD a, AccD b) { return AccD{a.v + b.v
 constexpr int kRedSegs = 6;
 constexpr int kRedLong = 48;
 constexpr int kRedThreads = 256;
-constexpr int kRedCtasPerSm = 8;
+constexpr int kRedCtasPerSm = 16;
 static_assert(kRedSegs * kCamPart <= kRedThreads && kPairPart <= kCamPart, "a group of lanes per row");
 
 // rows [p, p1) of a list, element el, in order
@@ -933,12 +935,16 @@ struct RedItem {
   const int* slots;
   const void* part;
   int begin, n, width;  // n = 0: nothing to do (its cluster is inactive, or no such item)
-  // element e of the sums: out[(e / 6) si + (e % 6) sc], negated for a pair
-  // block of a cluster of up to kMaxFreeSmall free images, which goes to its
-  // place in S (elimination order, lower triangle; and mirrored to out2)
+  // lane e of the sums goes to out[(e / 6) ld + e % 6].  The pair block of a
+  // cluster of up to kMaxFreeSmall free images goes negated to its place in the
+  // lower triangle of S (elimination order; and mirrored to out2): where that
+  // is the transposed block, lane e sums element (e % 6, e / 6), so that the
+  // stores stay in runs of six.
   double *out, *out2;
-  int si, sc;
+  int ld, trans;
 };
+// the element that lane e sums
+__device__ __forceinline__ int red_element(const RedItem& r, int e) { return r.trans ? (e % 6) * 6 + e / 6 : e; }
 __device__ __forceinline__ RedItem red_item(const BatchView& bv, int g, int mirror) {
   const int s = find_slot(bv.item_pre, bv.n, g);
   const DevCluster& C = bv.cl[s];
@@ -953,8 +959,8 @@ __device__ __forceinline__ RedItem red_item(const BatchView& bv, int g, int mirr
   r.slots = cam ? C.cam_slots : C.pair_slots;
   r.part = cam ? C.campart : C.pairpart;
   r.out2 = nullptr;
-  r.si = 6;
-  r.sc = 1;
+  r.ld = 6;
+  r.trans = 0;
   r.width = cam ? 39 : 36;
   if (cam) {
     r.out = C.camsum + (size_t)kCamPart * key;
@@ -967,8 +973,8 @@ __device__ __forceinline__ RedItem red_item(const BatchView& bv, int g, int mirr
     double* const rows_a = C.S + (size_t)pa * n + pb;
     double* const rows_b = C.S + (size_t)pb * n + pa;
     r.out = pa > pb ? rows_a : rows_b;
-    r.si = pa > pb ? n : 1;
-    r.sc = pa > pb ? 1 : n;
+    r.ld = n;
+    r.trans = pb > pa;
     if (mirror) r.out2 = pa > pb ? rows_b : rows_a;
     r.width = -36;
   }
@@ -977,12 +983,12 @@ __device__ __forceinline__ RedItem red_item(const BatchView& bv, int g, int mirr
 __device__ __forceinline__ void red_store(const RedItem& r, int el, double v) {
   const int i = el / 6, c = el - 6 * i;
   if (r.width < 0) v = -v;
-  r.out[(size_t)i * r.si + (size_t)c * r.sc] = v;
-  if (r.out2) r.out2[(size_t)i * r.sc + (size_t)c * r.si] = v;
+  r.out[(size_t)i * r.ld + c] = v;
+  if (r.out2) r.out2[(size_t)c * r.ld + i] = v;
 }
 
 template <typename Real>
-__global__ void __launch_bounds__(kRedThreads, 5) k_partial_reduce(BatchView bv, int mirror) {
+__global__ void __launch_bounds__(kRedThreads, 6) k_partial_reduce(BatchView bv, int mirror) {
   using Acc = typename AccOf<Real>::T;
   __shared__ typename Acc::Raw sums[2][kRedSegs][kCamPart];  // two items' worth: one barrier per long item
   __shared__ RedItem items[kRedSegs];
@@ -1002,7 +1008,7 @@ __global__ void __launch_bounds__(kRedThreads, 5) k_partial_reduce(BatchView bv,
     if (seg < group) {  // the short lists, a group each
       const RedItem r = items[seg];
       if (r.n > 0 && r.n <= kRedLong && el < abs(r.width)) {
-        const Real* part = (const Real*)r.part + el;
+        const Real* part = (const Real*)r.part + red_element(r, el);
         const int stride = abs(r.width) == 36 ? kPairPart : kCamPart;
         red_store(r, el, add_rows<Real>(part, stride, r.slots, r.begin, r.begin + r.n).get());
       }
@@ -1012,7 +1018,7 @@ __global__ void __launch_bounds__(kRedThreads, 5) k_partial_reduce(BatchView bv,
       if (r.n <= kRedLong) continue;
       const bool live = seg < kRedSegs && el < abs(r.width);
       if (live) {
-        const Real* part = (const Real*)r.part + el;
+        const Real* part = (const Real*)r.part + red_element(r, el);
         const int stride = abs(r.width) == 36 ? kPairPart : kCamPart;
         const int per = (r.n + kRedSegs - 1) / kRedSegs;
         const int p0 = r.begin + seg * per, p1 = r.begin + min(r.n, (seg + 1) * per);
