@@ -1715,8 +1715,7 @@ ba_status build_cluster(ba_ctx* ctx, const ba_cluster_desc* d, Cluster* c, const
   const size_t o_rhs = Lo.add(sizeof(double) * n);
   const size_t o_gc = Lo.add(sizeof(double) * n);
   const size_t o_Dc = Lo.add(sizeof(double) * n);
-  const size_t o_dc = Lo.add(sizeof(double) * n);
-  const size_t o_dc32 = Lo.add(sizeof(float) * n);
+  const size_t o_dcam = Lo.add(rs * kCamStep * (size_t)nc);
   const size_t o_tp = Lo.add(sizeof(double) * 2 * tiles.size());
   const size_t o_ptblk = Lo.add(rs * 16 * (size_t)np);
   const size_t o_trace = Lo.add(sizeof(StepRec) * kTraceCap);
@@ -1915,6 +1914,8 @@ ba_status build_cluster(ba_ctx* ctx, const ba_cluster_desc* d, Cluster* c, const
   h.n_cslots = n_cslots; h.n_pslots = n_pslots;
   h.sigma_px = d->sigma_px; h.huber_delta = d->huber_delta_px; h.sigma_gnss = d->sigma_gnss_m;
   h.sigma_imu = d->sigma_imu_rad;
+  h.inv_sigma = 1.0 / d->sigma_px;
+  h.half_inv_s2 = 0.5 / (d->sigma_px * d->sigma_px);
   h.inv_gnss2 = d->sigma_gnss_m > 0.0 ? 1.0 / (d->sigma_gnss_m * d->sigma_gnss_m) : 0.0;
   h.inv_imu2 = d->sigma_imu_rad > 0.0 ? 1.0 / (d->sigma_imu_rad * d->sigma_imu_rad) : 0.0;
   h.inv_sigma_f = (float)(1.0 / d->sigma_px);
@@ -1969,8 +1970,7 @@ ba_status build_cluster(ba_ctx* ctx, const ba_cluster_desc* d, Cluster* c, const
   h.rhs = (double*)(arena + o_rhs);
   h.gc = (double*)(arena + o_gc);
   h.Dc = (double*)(arena + o_Dc);
-  h.dc = (double*)(arena + o_dc);
-  h.dc32 = (float*)(arena + o_dc32);
+  h.dcam = arena + o_dcam;
   h.tilepart = (double*)(arena + o_tp);
   h.lm = (LmState*)(arena + o_lm);
   h.trace = (StepRec*)(arena + o_trace);

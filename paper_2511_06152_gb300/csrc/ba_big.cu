@@ -24,7 +24,7 @@
 //   k_big_solve_df   forward and backward substitution (one CTA, double-float,
 //                    the inverted diagonal blocks and the panels)
 //   k_big_resid      t = rhs - S x in binary64
-//   k_big_finish     dc, candidate poses, pred and prior terms, status
+//   k_big_finish     the images' steps, candidate poses, pred and prior terms, status
 //
 // Binary64 factorisation on the CUDA cores (BA_FLAG_BIG_FP64_FACTOR):
 //   (F = S)
@@ -322,19 +322,14 @@ __global__ void __launch_bounds__(256) k_big_resid(const DevCluster* dcl) {
   }
 }
 
-// dc (free-image order), candidate poses, pred and prior terms, status
+// candidate poses and the images' steps, pred and prior terms, status
 template <bool MIXED>
 __global__ void __launch_bounds__(512) k_big_finish(const DevCluster* dcl) {
   const DevCluster& C = *dcl;
   LmState* lm = C.lm;
-  const int n = 6 * C.n_free, tid = threadIdx.x;
+  const int tid = threadIdx.x;
   const bool fail = lm->pt_fail != 0 || *C.bflag != 0;
-  const double* x = C.bx + n;
-  for (int idx = tid; idx < n; idx += blockDim.x) {
-    const double v = fail ? 0.0 : x[6 * C.fpos[idx / 6] + idx % 6];
-    C.dc[idx] = v;
-    if (MIXED) C.dc32[idx] = (float)v;
-  }
+  const double* x = C.bx + 6 * C.n_free;
   double pc = 0.0, pn = 0.0;
   for (int k = tid; k < C.n_cams; k += blockDim.x) {
     double a, b;

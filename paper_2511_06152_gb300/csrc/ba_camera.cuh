@@ -1,5 +1,7 @@
 // Camera records and candidate poses, shared by the reduced-system solvers.
 #pragma once
+#include <type_traits>
+
 #include "ba_device.cuh"
 #include "ba_dfloat.cuh"
 #include "ba_internal.h"
@@ -70,6 +72,16 @@ __device__ inline void candidate_pose(const DevCluster& C, int k, const double* 
   }
 }
 
+// Entry q of the image's step for the back-substitution: dtheta and R^T dT (d:
+// the step, null for an image that keeps its pose; Rc: its current rotation)
+template <bool MIXED>
+__device__ __forceinline__ void store_cam_step(const DevCluster& C, int k, int q, const double* d, const double* Rc) {
+  using Real = typename std::conditional<MIXED, float, double>::type;
+  Real* o = reinterpret_cast<Real*>(C.dcam) + (size_t)kCamStep * k;
+  o[q] = d ? (Real)d[q] : Real(0);
+  o[4 + q] = d ? (Real)(Rc[q] * d[3] + Rc[3 + q] * d[4] + Rc[6 + q] * d[5]) : Real(0);
+}
+
 // The candidate to state buffer cur ^ 1 (and its double-float record in the
 // mixed path).
 template <bool MIXED>
@@ -91,6 +103,9 @@ __device__ inline void candidate_camera(const DevCluster& C, int k, const double
   candidate_pose(C, k, x, cur, fail, Rn, Tn);
   store_candidate<MIXED>(C, k, cur, Rn, Tn);
   const int f = C.free_idx[k];
+  for (int q = 0; q < 3; ++q)
+    store_cam_step<MIXED>(C, k, q, f >= 0 && !fail ? x + 6 * C.fpos[f] : nullptr,
+                          C.R + (size_t)cur * C.n_cams * 9 + 9 * k);
   *pc = 0.0;
   *pn = 0.0;
   if (f >= 0 && !fail) {

@@ -377,6 +377,49 @@ __device__ __forceinline__ bool obs_linearize(const Real* Rm, Real dx, Real dy, 
   return true;
 }
 
+// The point's share of one observation in the back-substitution, Jp^T (Jc dc),
+// from the image's step: with A = d(residual)/dXc, Jc dc = A (Xc x dtheta - R^T
+// dT) and Jp = A R^T, so that neither Jacobian is formed (and the robust weight
+// enters without its root).  d = X - T, dth = dtheta, dt = R^T dT.
+template <typename Real>
+__device__ __forceinline__ void obs_step(const Real* Rm, Real dx, Real dy, Real dz, const Real* in, Real uo, Real vo,
+                                         Real inv_sigma, Real delta, const Real dth[3], const Real dt[3], Real g[3]) {
+  const Real x = Rm[0] * dx + Rm[3] * dy + Rm[6] * dz;
+  const Real y = Rm[1] * dx + Rm[4] * dy + Rm[7] * dz;
+  const Real z = Rm[2] * dx + Rm[5] * dy + Rm[8] * dz;
+  const bool front = z > Real(kMinDepth);
+  const Real f = in[0], k1 = in[3], k2 = in[4], p1 = in[5], p2 = in[6];
+  const Real iz = recip_any(front ? z : Real(1));
+  const Real xn = x * iz, yn = y * iz;
+  const Real r2 = xn * xn + yn * yn;
+  const Real rad = Real(1) + r2 * (k1 + k2 * r2);
+  const Real xd = xn * rad + Real(2) * p1 * xn * yn + p2 * (r2 + Real(2) * xn * xn);
+  const Real yd = yn * rad + p1 * (r2 + Real(2) * yn * yn) + Real(2) * p2 * xn * yn;
+  const Real e0 = f * xd + in[1] - uo;
+  const Real e1 = f * yd + in[2] - vo;
+  const Real s = e0 * e0 + e1 * e1;
+  Real w = inv_sigma * inv_sigma;  // rho'(s) / sigma^2
+  if (s > delta * delta) w *= delta * rsqrt_any(s);
+  const Real drad = Real(2) * k1 + Real(4) * k2 * r2;
+  const Real D00 = rad + drad * xn * xn + Real(2) * p1 * yn + Real(6) * p2 * xn;
+  const Real D01 = drad * xn * yn + Real(2) * p1 * xn + Real(2) * p2 * yn;
+  const Real D11 = rad + drad * yn * yn + Real(6) * p1 * yn + Real(2) * p2 * xn;
+  // A = a (D | -D (xn, yn)^T), a = f / z
+  const Real c0 = y * dth[2] - z * dth[1] - dt[0];
+  const Real c1 = z * dth[0] - x * dth[2] - dt[1];
+  const Real c2 = x * dth[1] - y * dth[0] - dt[2];
+  const Real h0 = c0 - xn * c2, h1 = c1 - yn * c2;
+  const Real u0 = D00 * h0 + D01 * h1, u1 = D01 * h0 + D11 * h1;
+  Real b0 = D00 * u0 + D01 * u1, b1 = D01 * u0 + D11 * u1;
+  const Real a = f * iz;
+  const Real m = front ? w * a * a : Real(0);
+  b0 *= m;
+  b1 *= m;
+  const Real b2 = -(xn * b0 + yn * b1);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) g[i] = Rm[3 * i] * b0 + Rm[3 * i + 1] * b1 + Rm[3 * i + 2] * b2;
+}
+
 // The LM decision of one cluster once every tile of its back-substitution is
 // done, by one thread: gain ratio from F(x + d) and pred (Fo, pp: the sums of
 // the tiles' cost and pred terms), accept or reject, Nielsen's update of mu and

@@ -580,6 +580,7 @@ __device__ __noinline__ void candidate_quad(const DevCluster& C, int k, const do
     for (int c = 0; c < 3; ++c) Rn[c] = row[c];
     C.T[(size_t)(cur ^ 1) * nc * 3 + 3 * k + q] = t;
     if constexpr (MIXED) write_camdf_row(C, cur ^ 1, k, q, row, t);
+    store_cam_step<MIXED>(C, k, q, moves ? x + 6 * C.fpos[f] : nullptr, Rc);
     return;
   }
   double v = 0.0;
@@ -807,11 +808,6 @@ __global__ void __cluster_dims__(kFC, 1, 1) __launch_bounds__(kFactorMaxThreads)
     cl.sync();
     if (rank == 0) {
       for (int idx = tid; idx < 4 * nc; idx += bs) candidate_quad<MIXED>(C, idx >> 2, S.x, cur, bad, idx & 3, true, nullptr);
-      for (int idx = tid; idx < n; idx += bs) {  // back to free-image order
-        const double v = S.x[6 * C.fpos[idx / 6] + idx % 6];
-        C.dc[idx] = v;
-        if (MIXED) C.dc32[idx] = (float)v;
-      }
       if (tid == 0) {
         lm->status = lm->dev_error ? lm->dev_error : (bad ? BA_STATUS_NOT_PD : 0);
         lm->dev_error = 0;

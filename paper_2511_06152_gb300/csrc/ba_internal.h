@@ -49,6 +49,7 @@ constexpr int kCostInitThreads = 256;  // threads of k_cost_init's CTA (its sums
 // the low words of R [24, 33), f.lo 33, k1 k2 p1 p2 .lo [34, 38), pad to 40
 constexpr int kCamDf = 40;
 constexpr int kCamReal = 20;
+constexpr int kCamStep = 8;
 
 struct Tile {
   int obs_begin;
@@ -118,6 +119,7 @@ struct DevCluster {
   int n_tiles, n_chunks, n_pairs, n_cslots, n_pslots, pad_i;
   double sigma_px, huber_delta, sigma_gnss, sigma_imu;
   double inv_gnss2, inv_imu2;  // 1 / sigma^2 of the priors, 0 when off
+  double inv_sigma, half_inv_s2;  // 1 / sigma_px, 1 / (2 sigma_px^2)
   float inv_sigma_f, delta_f, half_inv_s2_f, pad_f;  // binary32 copies of 1/sigma_px, delta, 1/(2 sigma_px^2)
 
   const double* intr;      // [nc][7]
@@ -187,8 +189,9 @@ struct DevCluster {
   double* rhs;      // [n]
   double* gc;       // [n]
   double* Dc;       // [n]
-  double* dc;       // [n]
-  float* dc32;      // [n] binary32 copy of dc (mixed path)
+  // The step of every image for the back-substitution, Real [nc][kCamStep]:
+  // dtheta 0 .. 2, R^T dT 4 .. 6 (zero for a fixed image)
+  void* dcam;
   double* tilepart; // [n_tiles][2]: cost, point pred (or max |g_p| in the diagnostic pass)
   LmState* lm;
   StepRec* trace;   // [trace_cap]

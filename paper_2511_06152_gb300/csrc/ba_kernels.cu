@@ -209,7 +209,7 @@ __device__ __forceinline__ void ld4(const double* r, int at, double* o) {
 }
 
 // What one lane knows after linearising its observation of a tile: the
-// whitened, robust-weighted Jacobians and residual, Z = Jc^T Jp L^-T, and
+// whitened, robust-weighted Jacobians and residual, P = Jp L^-T, and
 // (broadcast from the point's first lane) L^-1 and q = L^-1 g_p of the damped
 // point block; D_p and g_p are valid on the point's first lane.
 template <bool MIXED>
@@ -217,16 +217,16 @@ struct TileLin {
   using Real = typename RealOf<MIXED>::T;
   bool act, head;
   int o, k, j, seg_start, seg_end, span;
-  Real Jc[12], r0, r1, Z[18];
+  Real Jc[12], r0, r1;
   Real P[6];  // P = Jp M^T (2x3, row-major), so that Z = Jc^T P
   Real m00, m10, m11, m20, m21, m22, q0, q1, q2;
   Real d0, d1, d2, g0, g1, g2;
 };
 
 // Where the mixed linearisation reads a chunk's observations (camera, point,
-// observation relative to the principal point) and the current points:
-// the cluster's arrays in global memory, or a shared-memory copy of the
-// chunk's ranges (index o - o0, point j - j0).
+// observation relative to the principal point) and the current points: a
+// shared-memory copy of the chunk's ranges (index o - o0, point j - j0), the
+// points of a chunk that spans too many in global memory.
 struct ObsView {
   const int* cam;
   const int* pt;
@@ -235,17 +235,8 @@ struct ObsView {
   int o0, j0;
 };
 
-__device__ __forceinline__ ObsView global_view(const DevCluster& C, int cur) {
-  return ObsView{C.obs_cam, C.obs_pt, C.obs_chi, reinterpret_cast<const float2*>(C.X) + (size_t)cur * C.n_pts * 3,
-                 0, 0};
-}
-
-// Linearise one tile (one warp).  The same arithmetic wherever it is called
-// (the back-substitution linearises again rather than storing the result).
-// PT_BUF: the point blocks' M, q, D_p and g_p are read from C.ptblk, where
-// the linearise+Schur kernel of the same iteration stored them (same values),
-// instead of being reduced and factored again.
-template <bool MIXED, bool WANT_Z = true, bool PT_BUF = false>
+// Linearise one tile (one warp).
+template <bool MIXED>
 __device__ __forceinline__ void linearize_tile(const DevCluster& C, LmState* lm, const Tile& tl, int lane,
                                                bool report_fail, TileLin<MIXED>& L, const ObsView& V) {
   using Real = typename RealOf<MIXED>::T;
@@ -269,7 +260,7 @@ __device__ __forceinline__ void linearize_tile(const DevCluster& C, LmState* lm,
     delta = C.delta_f;
   } else {
     mu = lm->mu;
-    inv_sigma = 1.0 / C.sigma_px;
+    inv_sigma = C.inv_sigma;
     delta = C.huber_delta;
   }
   Real Jp[6];
@@ -286,9 +277,9 @@ __device__ __forceinline__ void linearize_tile(const DevCluster& C, LmState* lm,
       const CamDf cd = load_camdf_lin(camdf_ptr(C, cur, L.k));
       const float2* xp = V.x + (size_t)(L.j - V.j0) * 3;
       const float2 a = xp[0], b = xp[1], c = xp[2];
-      dx = df_to_f(df_sub(dfl{a.x, a.y}, cd.T[0]));
-      dy = df_to_f(df_sub(dfl{b.x, b.y}, cd.T[1]));
-      dz = df_to_f(df_sub(dfl{c.x, c.y}, cd.T[2]));
+      dx = df_sum_to_f(dfl{a.x, a.y}, df_neg(cd.T[0]));
+      dy = df_sum_to_f(dfl{b.x, b.y}, df_neg(cd.T[1]));
+      dz = df_sum_to_f(dfl{c.x, c.y}, df_neg(cd.T[2]));
 #pragma unroll
       for (int i = 0; i < 9; ++i) Rm[i] = cd.R[i].hi;
       in[0] = cd.f.hi; in[1] = 0.f; in[2] = 0.f;
@@ -314,17 +305,7 @@ __device__ __forceinline__ void linearize_tile(const DevCluster& C, LmState* lm,
       for (int i = 0; i < 12; ++i) L.Jc[i] = 0;
     }
   }
-  if constexpr (PT_BUF) {
-    // every lane of a point reads its block (one address per point); an
-    // inactive lane reads point 0 and keeps P = 0 (its Jp is 0)
-    const Real* pb = reinterpret_cast<const Real*>(C.ptblk) + (size_t)(L.act ? L.j : 0) * 16;
-    Real w[16];
-    ld4(pb, 0, w); ld4(pb, 4, w + 4); ld4(pb, 8, w + 8); ld4(pb, 12, w + 12);
-    L.m00 = w[0]; L.m10 = w[1]; L.m11 = w[2]; L.m20 = w[3]; L.m21 = w[4]; L.m22 = w[5];
-    L.q0 = w[6]; L.q1 = w[7]; L.q2 = w[8];
-    L.d0 = w[9]; L.d1 = w[10]; L.d2 = w[11];
-    L.g0 = w[12]; L.g1 = w[13]; L.g2 = w[14];
-  } else {
+  {
     // point blocks by segmented reduction
     Real v00 = Jp[0] * Jp[0] + Jp[3] * Jp[3];
     Real v01 = Jp[0] * Jp[1] + Jp[3] * Jp[4];
@@ -381,7 +362,7 @@ __device__ __forceinline__ void linearize_tile(const DevCluster& C, LmState* lm,
     L.q1 = __shfl_sync(BA_FULL_MASK, q1, L.seg_start);
     L.q2 = __shfl_sync(BA_FULL_MASK, q2, L.seg_start);
   }
-  // P = Jp M^T (2x3), Z = Jc^T P (6x3)
+  // P = Jp M^T (2x3), so that Z = Jc^T P (6x3)
   const Real P00 = Jp[0] * L.m00;
   const Real P01 = Jp[0] * L.m10 + Jp[1] * L.m11;
   const Real P02 = Jp[0] * L.m20 + Jp[1] * L.m21 + Jp[2] * L.m22;
@@ -390,14 +371,6 @@ __device__ __forceinline__ void linearize_tile(const DevCluster& C, LmState* lm,
   const Real P12 = Jp[3] * L.m20 + Jp[4] * L.m21 + Jp[5] * L.m22;
   L.P[0] = P00; L.P[1] = P01; L.P[2] = P02;
   L.P[3] = P10; L.P[4] = P11; L.P[5] = P12;
-  if constexpr (WANT_Z) {
-#pragma unroll
-    for (int m = 0; m < 6; ++m) {
-      L.Z[3 * m + 0] = L.Jc[m] * P00 + L.Jc[6 + m] * P10;
-      L.Z[3 * m + 1] = L.Jc[m] * P01 + L.Jc[6 + m] * P11;
-      L.Z[3 * m + 2] = L.Jc[m] * P02 + L.Jc[6 + m] * P12;
-    }
-  }
 }
 
 // ------------------------------------------------------------------ K1: linearise + Schur reductions, one CTA per chunk
@@ -761,7 +734,7 @@ __global__ void __launch_bounds__(kChunkThreads, MIXED ? kLinSchurMinBlocksMixed
           tl = C.tiles[ch.tile_begin + t];
         }
         TileLin<MIXED> L;
-        linearize_tile<MIXED, false>(C, lm, tl, lane, true, L, V);
+        linearize_tile<MIXED>(C, lm, tl, lane, true, L, V);
         if (L.act) st_rec<MIXED>(srec + (size_t)(L.o - ch.obs_begin) * kSrec, L);
         if (L.head) st_ptblk<MIXED>(C, L);
         if (diag) {  // largest |g_p| of the tile, for the gradient norm
@@ -1115,54 +1088,71 @@ __device__ void backsub_tile(const DevCluster& C, LmState* lm, int local, int la
   using Real = typename RealOf<MIXED>::T;
   {
     const Tile tl = C.tiles[local];
-    TileLin<MIXED> L;
-    linearize_tile<MIXED, false, true>(C, lm, tl, lane, false, L, global_view(C, lm->cur));
+    const bool act = lane < tl.n_obs;
+    const int o = tl.obs_begin + (act ? lane : 0);
+    const int k = act ? C.obs_cam[o] : 0, j = act ? C.obs_pt[o] : -1 - lane;
+    int seg_start, seg_end;
+    segments(j, lane, seg_start, seg_end);
+    const int span = segment_span(seg_start, seg_end);
+    const bool head = act && lane == seg_start;
     const int cur = lm->cur;
-    Real mu_r;
-    if constexpr (MIXED) mu_r = lm->mu_f; else mu_r = lm->mu;
-    // t = Z^T dc_k = P^T (Jc dc_k)
-    Real t0 = 0, t1 = 0, t2 = 0;
-    const int f = L.act ? C.free_idx[L.k] : -1;
-    if (f >= 0) {
-      Real d[6];
+    // this observation's share of Jp^T (Jc dc)
+    Real t[3] = {0, 0, 0};
+    if (act) {
+      const Real* st = reinterpret_cast<const Real*>(C.dcam) + (size_t)kCamStep * k;
+      Real dth[4], dt[4];
+      ld4(st, 0, dth);
+      ld4(st, 4, dt);
+      Real Rm[9], in[7];
       if constexpr (MIXED) {
-        const float2* d2 = reinterpret_cast<const float2*>(C.dc32 + 6 * f);
-        const float2 u0 = d2[0], u1 = d2[1], u2 = d2[2];
-        d[0] = u0.x; d[1] = u0.y; d[2] = u1.x; d[3] = u1.y; d[4] = u2.x; d[5] = u2.y;
+        const CamDf cd = load_camdf_lin(camdf_ptr(C, cur, k));
+        const float2* xp = xdf_ptr(C, cur, j);
+        const float2 a = xp[0], b = xp[1], c = xp[2];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) Rm[i] = cd.R[i].hi;
+        in[0] = cd.f.hi; in[1] = 0.f; in[2] = 0.f;
+        in[3] = cd.k1.hi; in[4] = cd.k2.hi; in[5] = cd.p1.hi; in[6] = cd.p2.hi;
+        const float2 ch = C.obs_chi[o];
+        obs_step<Real>(Rm, df_sum_to_f(dfl{a.x, a.y}, df_neg(cd.T[0])), df_sum_to_f(dfl{b.x, b.y}, df_neg(cd.T[1])),
+                       df_sum_to_f(dfl{c.x, c.y}, df_neg(cd.T[2])), in, ch.x, ch.y, C.inv_sigma_f, C.delta_f, dth, dt, t);
       } else {
+        const double* cr = (const double*)C.camreal + (size_t)kCamReal * k;
 #pragma unroll
-        for (int m = 0; m < 6; ++m) d[m] = C.dc[6 * f + m];
-      }
-      Real u0 = 0, u1 = 0;
+        for (int i = 0; i < 9; ++i) Rm[i] = cr[i];
 #pragma unroll
-      for (int m = 0; m < 6; ++m) {
-        u0 += L.Jc[m] * d[m];
-        u1 += L.Jc[6 + m] * d[m];
+        for (int i = 0; i < 7; ++i) in[i] = cr[12 + i];
+        const double* Xd = C.X + ((size_t)cur * C.n_pts + j) * 3;
+        const double2 u = reinterpret_cast<const double2*>(C.obs_uv)[o];
+        obs_step<Real>(Rm, Xd[0] - cr[9], Xd[1] - cr[10], Xd[2] - cr[11], in, u.x, u.y, C.inv_sigma, C.huber_delta,
+                       dth, dt, t);
       }
-      t0 = L.P[0] * u0 + L.P[3] * u1;
-      t1 = L.P[1] * u0 + L.P[4] * u1;
-      t2 = L.P[2] * u0 + L.P[5] * u1;
     }
-    t0 = seg_reduce(t0, lane, L.seg_start, L.seg_end, L.span);
-    t1 = seg_reduce(t1, lane, L.seg_start, L.seg_end, L.span);
-    t2 = seg_reduce(t2, lane, L.seg_start, L.seg_end, L.span);
-    // head: dX = M^T (q - t), candidate point, pred term
+#pragma unroll
+    for (int i = 0; i < 3; ++i) t[i] = seg_reduce(t[i], lane, seg_start, seg_end, span);
+    // head: dX = M^T M (g_p - t), candidate point, pred term (M, D_p and g_p as
+    // the linearise+Schur kernel of this iteration left them; the difference is
+    // taken before M, where it cancels exactly)
     Real dX0 = 0, dX1 = 0, dX2 = 0;
     Real pp = 0;  // dX^T (mu Dp dX + gp)
-    if (L.head) {
-      const Real v0 = L.q0 - t0, v1 = L.q1 - t1, v2 = L.q2 - t2;
-      dX0 = L.m00 * v0 + L.m10 * v1 + L.m20 * v2;
-      dX1 = L.m11 * v1 + L.m21 * v2;
-      dX2 = L.m22 * v2;
-      pp = dX0 * (mu_r * L.d0 * dX0 + L.g0) + dX1 * (mu_r * L.d1 * dX1 + L.g1) + dX2 * (mu_r * L.d2 * dX2 + L.g2);
+    if (head) {
+      const Real* pb = reinterpret_cast<const Real*>(C.ptblk) + (size_t)j * 16;
+      Real w[16];  // m00 m10 m11 m20 m21 m22 q0 q1 q2 d0 d1 d2 g0 g1 g2
+      ld4(pb, 0, w); ld4(pb, 4, w + 4); ld4(pb, 8, w + 8); ld4(pb, 12, w + 12);
+      Real mu;
+      if constexpr (MIXED) mu = lm->mu_f; else mu = lm->mu;
+      const Real s0 = w[12] - t[0], s1 = w[13] - t[1], s2 = w[14] - t[2];
+      const Real v0 = w[0] * s0;
+      const Real v1 = w[1] * s0 + w[2] * s1;
+      const Real v2 = w[3] * s0 + w[4] * s1 + w[5] * s2;
+      dX0 = w[0] * v0 + w[1] * v1 + w[3] * v2;
+      dX1 = w[2] * v1 + w[4] * v2;
+      dX2 = w[5] * v2;
+      pp = dX0 * (mu * w[9] * dX0 + w[12]) + dX1 * (mu * w[10] * dX1 + w[13]) + dX2 * (mu * w[11] * dX2 + w[14]);
     }
-    const int o = L.o, k = L.k, j = L.j;
-    const bool act = L.act;
-    const int seg_start = L.seg_start;
     double cost = 0.0;
     if constexpr (MIXED) {
       dfl x0{0.f, 0.f}, x1{0.f, 0.f}, x2{0.f, 0.f};
-      if (L.head) {
+      if (head) {
         const float2* xp = xdf_ptr(C, cur, j);
         const float2 a = xp[0], b = xp[1], c = xp[2];
         x0 = df_add_f(dfl{a.x, a.y}, dX0);
@@ -1193,7 +1183,7 @@ __device__ void backsub_tile(const DevCluster& C, LmState* lm, int local, int la
       if (lane == 0) cost = df_to_d(cst);
     } else {
       double x0 = 0.0, x1 = 0.0, x2 = 0.0;
-      if (L.head) {
+      if (head) {
         const double* X = C.X + ((size_t)cur * C.n_pts + j) * 3;
         x0 = X[0] + (double)dX0;
         x1 = X[1] + (double)dX1;
@@ -1209,7 +1199,7 @@ __device__ void backsub_tile(const DevCluster& C, LmState* lm, int local, int la
         const double* Rn = C.R + ((size_t)(cur ^ 1) * C.n_cams + k) * 9;
         const double* Tn = C.T + ((size_t)(cur ^ 1) * C.n_cams + k) * 3;
         const double2 u = reinterpret_cast<const double2*>(C.obs_uv)[o];
-        cost = obs_cost(Rn, Tn, C.intr + 7 * k, Xn, u.x, u.y, 0.5 / (C.sigma_px * C.sigma_px), C.huber_delta);
+        cost = obs_cost(Rn, Tn, C.intr + 7 * k, Xn, u.x, u.y, C.half_inv_s2, C.huber_delta);
       }
       cost = warp_sum(cost);
     }
@@ -1270,7 +1260,7 @@ __global__ void __launch_bounds__(256) k_cost_tiles(BatchView bv) {
         const double2 u = reinterpret_cast<const double2*>(C.obs_uv)[o];
         cost = obs_cost(C.R + ((size_t)cur * C.n_cams + k) * 9, C.T + ((size_t)cur * C.n_cams + k) * 3,
                         C.intr + 7 * k, C.X + ((size_t)cur * C.n_pts + j) * 3, u.x, u.y,
-                        0.5 / (C.sigma_px * C.sigma_px), C.huber_delta);
+                        C.half_inv_s2, C.huber_delta);
       }
       cost = warp_sum(cost);
     }
