@@ -2490,32 +2490,33 @@ BA_API ba_status ba_footprints(ba_ctx* ctx, int32_t n, const double* intr, doubl
   if (n == 0) return BA_OK;
   std::lock_guard<std::mutex> g(ctx->api_mu);
   const size_t nh = (size_t)dsm->nx * dsm->ny;
-  DsmView D{dsm->nx, dsm->ny, dsm->x0, dsm->y0, dsm->dx, dsm->dy, dsm->h[0], dsm->h[0], nullptr};
-  for (size_t i = 0; i < nh; ++i) {
-    if (!std::isfinite(dsm->h[i])) return set_err(ctx, BA_ERR_INVALID, "ba_footprints: non-finite DSM height");
-    D.hmin = std::min(D.hmin, dsm->h[i]);
-    D.hmax = std::max(D.hmax, dsm->h[i]);
-  }
+  DsmView D{dsm->nx, dsm->ny, dsm->x0, dsm->y0, dsm->dx, dsm->dy, nullptr};
   const size_t b_in = sizeof(double) * (size_t)n * (7 + 9 + 3), b_h = sizeof(double) * nh,
                b_out = sizeof(double) * (size_t)n * 12;
   char* buf = nullptr;
-  CUDA_TRY(ctx, scratch_alloc(ctx, (void**)&buf, b_in + b_h + b_out));
+  CUDA_TRY(ctx, scratch_alloc(ctx, (void**)&buf, b_in + b_h + b_out + sizeof(long long) * kRangeWords));
   double* d_intr = (double*)buf;
   double* d_R = d_intr + 7 * (size_t)n;
   double* d_T = d_R + 9 * (size_t)n;
   double* d_h = d_T + 3 * (size_t)n;
   double* d_out = d_h + nh;
+  long long* d_range = (long long*)(d_out + 12 * (size_t)n);
   CUDA_TRY(ctx, cudaMemcpyAsync(d_intr, intr, sizeof(double) * 7 * n, cudaMemcpyHostToDevice, ctx->stream));
   CUDA_TRY(ctx, cudaMemcpyAsync(d_R, R, sizeof(double) * 9 * n, cudaMemcpyHostToDevice, ctx->stream));
   CUDA_TRY(ctx, cudaMemcpyAsync(d_T, T, sizeof(double) * 3 * n, cudaMemcpyHostToDevice, ctx->stream));
   CUDA_TRY(ctx, cudaMemcpyAsync(d_h, dsm->h, b_h, cudaMemcpyHostToDevice, ctx->stream));
   D.h = d_h;
-  launch_footprints(n, d_intr, width, height, d_R, d_T, D, d_out, ctx->stream);
+  launch_footprints(n, d_intr, width, height, d_R, d_T, D, d_range, d_out, ctx->stream);
   note_direct(ctx);
-  CUDA_TRY(ctx, cudaMemcpyAsync(corners, d_out, b_out, cudaMemcpyDeviceToHost, ctx->stream));
+  long long range[kRangeWords] = {0, 0, 0};
+  CUDA_TRY(ctx, cudaMemcpyAsync(range, d_range, sizeof(range), cudaMemcpyDeviceToHost, ctx->stream));
+  CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
+  // the corners of a raster that is not finite are not handed out
+  if (!range[2]) CUDA_TRY(ctx, cudaMemcpyAsync(corners, d_out, b_out, cudaMemcpyDeviceToHost, ctx->stream));
   CUDA_TRY(ctx, cudaFreeAsync(buf, ctx->stream));
   CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
   CUDA_TRY(ctx, cudaGetLastError());
+  if (range[2]) return set_err(ctx, BA_ERR_INVALID, "ba_footprints: non-finite DSM height");
   return BA_OK;
 }
 
