@@ -507,7 +507,8 @@ BA_API ba_status ba_cost_noalloc(const ba_cluster_desc* d, void* stream, double*
  * Launch and presort parameters of the LM iteration.  None changes what is
  * computed; chunk_tiles changes the order of some sums (every
  * configuration is deterministic: alone = in a batch, bit for bit).
- * Values: chunk_tiles 0 (the precision's maximum: 16 mixed, 8 FP64) or
+ * Values: chunk_tiles 0 (by the cluster's size: the precision's maximum, 16
+ * mixed and 8 FP64, or fewer for a cluster that would not cover the SMs) or
  * 4 .. that maximum; lin_ctas_per_sm and back_ctas_per_sm 1 .. 32;
  * factor_nb 2 .. 32; factor_threads 256, 384 or 512; big_panel_w 1, 2, 4, 8,
  * 16 or 32; batch_chains 1 .. 8.  ms_default / ms_tuned: what ba_autotune measured (device time

@@ -553,6 +553,7 @@ ba_status get_plan(ba_ctx* ctx, const std::vector<ba_cluster_id>& ids, Plan** ou
   p->bv.total_items = pre[2 * (n + 1) + n];
   p->bv.max_n = max_n;
   p->bv.inject = ctx->inject;
+  for (BigRef& b : p->big) b.early = chh.empty();
   apply_tune(ctx, p->bv);
   for (const ChainHost& h : chh) {
     const int m = (int)h.mem.size();
@@ -1272,7 +1273,7 @@ ba_status build_cluster(ba_ctx* ctx, const ba_cluster_desc* d, Cluster* c, const
   // chunk the observation lists of its free cameras and the observation pairs
   // of its co-visible camera pairs (all in increasing point-major order)
   const bool mixed = ctx->mixed;
-  const int ch_tiles = ctx->tune.chunk_tiles > 0 ? ctx->tune.chunk_tiles : chunk_tiles(mixed);
+  const int ch_tiles = ctx->tune.chunk_tiles > 0 ? ctx->tune.chunk_tiles : default_chunk_tiles((int)tiles.size(), nf, mixed);
   std::vector<Chunk> chunks;
   for (size_t t = 0; t < tiles.size();) {
     Chunk ch{};

@@ -100,6 +100,8 @@ __global__ void k_big_prior(const DevCluster* dcl) {
 
 // S(a, b) = -sum Z_a Z_b^T for every co-visible pair, both triangles
 __global__ void k_big_pairs(const DevCluster* dcl) {
+  dependency_wait();
+  dependency_trigger();
   const DevCluster& C = *dcl;
   const int n = 6 * C.n_free;
   for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < C.n_pairs * 36; idx += gridDim.x * blockDim.x) {
@@ -309,6 +311,8 @@ __global__ void __launch_bounds__(1024) k_big_solve(const DevCluster* dcl, int m
 
 // t = rhs - S x over the envelope (warp per row)
 __global__ void __launch_bounds__(256) k_big_resid(const DevCluster* dcl) {
+  dependency_wait();
+  dependency_trigger();
   const DevCluster& C = *dcl;
   const int n = 6 * C.n_free, lane = threadIdx.x & 31;
   const double* x = C.bx + n;
@@ -325,6 +329,8 @@ __global__ void __launch_bounds__(256) k_big_resid(const DevCluster* dcl) {
 // candidate poses and the images' steps, pred and prior terms, status
 template <bool MIXED>
 __global__ void __launch_bounds__(512) k_big_finish(const DevCluster* dcl) {
+  dependency_wait();
+  dependency_trigger();
   const DevCluster& C = *dcl;
   LmState* lm = C.lm;
   const int tid = threadIdx.x;
@@ -375,6 +381,8 @@ __device__ __forceinline__ float* df_lo(const DevCluster& C) {
 // F = S on the lower triangle as double-float (entries outside the envelope
 // are zero in S and become zero here), one CTA per row.
 __global__ void __launch_bounds__(256) k_big_split(const DevCluster* dcl) {
+  dependency_wait();
+  dependency_trigger();
   const DevCluster& C = *dcl;
   const int n = 6 * C.n_free;
   float* Fh = df_hi(C);
@@ -411,6 +419,8 @@ constexpr int kPld = kBigNB + 1;  // padded leading dimension of the shared bloc
 // with warp-level synchronisation only, then the whole CTA applies the
 // block's rank-pw update below it: two block-wide barriers per block.
 __global__ void __launch_bounds__(kPanelThreads) k_big_panel(const DevCluster* dcl, int k, int pw) {
+  dependency_wait();
+  dependency_trigger();
   const DevCluster& C = *dcl;
   const int n = 6 * C.n_free, r0 = kBigNB * k, nb = min(kBigNB, n - r0);
   float* Fh = df_hi(C);
@@ -584,7 +594,11 @@ __global__ void __launch_bounds__(kUpdThreads, 1) k_big_update_tc(const DevClust
   const int R0 = kBigNB * (k + 1), band_end = min(n, R0 + kBigNB * m);
   const int jb = blockIdx.x, rg = blockIdx.y;
   const int rA = R0 + kUpdM * rg, cB = R0 + kUpdN * jb;
-  if (rA >= band_end || rA + kUpdM - 1 < cB) return;  // past the band, or above the diagonal
+  if (rA >= band_end || rA + kUpdM - 1 < cB) {  // past the band, or above the diagonal
+    dependency_wait();
+    dependency_trigger();
+    return;
+  }
   extern __shared__ __align__(1024) unsigned char smu[];
   unsigned char* sa = smu;
   unsigned char* sb = smu + (size_t)kSlices * kUpdA;
@@ -599,6 +613,8 @@ __global__ void __launch_bounds__(kUpdThreads, 1) k_big_update_tc(const DevClust
     fence_barrier_init();
   }
   if (warp == 0) tmem_alloc(s_tmem, kUpdTmemCols);
+  dependency_wait();
+  dependency_trigger();
   if (tid < kUpdN) s_ecol[tid] = C.dexp[cB + tid];
   tc_fence_before();
   __syncthreads();
@@ -690,6 +706,8 @@ constexpr int kSolveChunk = 12;  // entries a lane loads before it sums them
 // groups of kSolveChunk before it sums them.  x = S^-1 rhs (mode 0) or
 // x += S^-1 t (mode 1), binary64 in and out.
 __global__ void __launch_bounds__(1024) k_big_solve_df(const DevCluster* dcl, int mode) {
+  dependency_wait();
+  dependency_trigger();
   const DevCluster& C = *dcl;
   extern __shared__ float sv[];
   const int n = 6 * C.n_free, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -822,20 +840,20 @@ void launch_big_solve(const BigRef& b, bool mixed, int refine_steps, int assembl
   if (assemble_only) return;
   const int nblk = (n + kBigNB - 1) / kBigNB;
   if (b.tc) {
-    LAUNCH(KK_FACTOR, st, k_big_split<<<std::min(n, num_sms() * 8), 256, 0, st>>>(b.d));
+    LAUNCH(KK_FACTOR, st, launch_dependent(b.early, k_big_split, std::min(n, num_sms() * 8), 256, 0, st, b.d));
     for (int k = 0; k < nblk; ++k) {
       const int m = b.below[k];
-      LAUNCH(KK_FACTOR, st, k_big_panel<<<1 + m, kPanelThreads, 0, st>>>(b.d, k, b.panel_w));
+      LAUNCH(KK_FACTOR, st, launch_dependent(b.early, k_big_panel, 1 + m, kPanelThreads, 0, st, b.d, k, b.panel_w));
       if (m > 0) {
         const dim3 grid(m, (kBigNB * m + kUpdM - 1) / kUpdM);
-        LAUNCH(KK_FACTOR, st, k_big_update_tc<<<grid, kUpdThreads, kUpdSmem, st>>>(b.d, k, m));
+        LAUNCH(KK_FACTOR, st, launch_dependent(b.early, k_big_update_tc, grid, kUpdThreads, kUpdSmem, st, b.d, k, m));
       }
     }
     const size_t sm = big_solve_df_smem(n);
-    LAUNCH(KK_FACTOR, st, k_big_solve_df<<<1, 1024, sm, st>>>(b.d, 0));
+    LAUNCH(KK_FACTOR, st, launch_dependent(b.early, k_big_solve_df, 1, 1024, sm, st, b.d, 0));
     for (int it = 0; it < refine_steps; ++it) {
-      LAUNCH(KK_FACTOR, st, k_big_resid<<<grid_for_big(n * 32, 256), 256, 0, st>>>(b.d));
-      LAUNCH(KK_FACTOR, st, k_big_solve_df<<<1, 1024, sm, st>>>(b.d, 1));
+      LAUNCH(KK_FACTOR, st, launch_dependent(b.early, k_big_resid, grid_for_big(n * 32, 256), 256, 0, st, b.d));
+      LAUNCH(KK_FACTOR, st, launch_dependent(b.early, k_big_solve_df, 1, 1024, sm, st, b.d, 1));
     }
   } else {
     cudaMemcpyAsync(b.F, b.S, nn * sizeof(double), cudaMemcpyDeviceToDevice, st);
@@ -854,8 +872,8 @@ void launch_big_solve(const BigRef& b, bool mixed, int refine_steps, int assembl
       LAUNCH(KK_FACTOR, st, k_big_solve<<<1, 1024, sm, st>>>(b.d, 1));
     }
   }
-  if (mixed) LAUNCH(KK_FACTOR, st, k_big_finish<true><<<1, 512, 0, st>>>(b.d));
-  else LAUNCH(KK_FACTOR, st, k_big_finish<false><<<1, 512, 0, st>>>(b.d));
+  LAUNCH(KK_FACTOR, st,
+         launch_dependent(b.early, mixed ? k_big_finish<true> : k_big_finish<false>, 1, 512, 0, st, b.d));
 }
 
 cudaError_t set_big_attributes(int max_n) {

@@ -624,7 +624,6 @@ __global__ void __cluster_dims__(kFC, 1, 1) __launch_bounds__(kFactorMaxThreads)
     const bool keep_s = refine_steps > 0;  // S in binary64 in global memory, for the refinement
 
     // ---- assembly (the images in elimination order: position p = fpos[f])
-    if (rank == 0 && tid == 0) lm->tiles_done = 0;  // the back-substitution counts its tiles from here
     if (tid == 0) {
       fail = lm->pt_fail;
       next[0] = next[1] = 0;
@@ -634,11 +633,12 @@ __global__ void __cluster_dims__(kFC, 1, 1) __launch_bounds__(kFactorMaxThreads)
       prior_quad(C, C.cam_of_free[f], C.R + (size_t)cur * nc * 9, C.T + (size_t)cur * nc * 3, idx & 3,
                  pr + kPr * C.fpos[f]);
     }
+    for (int b = tid; b < nb; b += bs) S.blkfirst[b] = 6 * C.env_first[(8 * b) / 6] / 8;
     for (int idx = tid; idx < nf * 39; idx += bs) {
       const int f = idx / 39, e = idx - 39 * f;
       cd[40 * C.fpos[f] + e] = C.camsum[(size_t)kCamPart * f + e];
     }
-    for (int b = tid; b < nb; b += bs) S.blkfirst[b] = 6 * C.env_first[(8 * b) / 6] / 8;
+    if (rank == 0 && tid == 0) lm->tiles_done = 0;  // the back-substitution counts its tiles from here
     __syncthreads();
     // damping, gradient, right-hand side; the scale of each row
     for (int i = tid; i < n8; i += bs) {

@@ -276,6 +276,36 @@ struct LaunchScope {
 
 int num_sms();
 
+// Programmatic dependent launch: a kernel of the global-memory solver's chain
+// may be scheduled while its predecessor on the stream still runs.  Every
+// kernel launched so waits for its predecessor's end (dependency_wait) before
+// it reads what earlier kernels wrote, and only then lets its own successor be
+// scheduled (dependency_trigger): when a kernel starts, everything up to its
+// predecessor's predecessor has ended.  Both are without effect in a kernel
+// launched the usual way.  (An iteration's other kernels gained nothing by it:
+// 24 images 3.39 against 3.42 ms per 20 iterations, but 12 images 0.94
+// against 0.91 ms per 10 and serving 16 windows 6.62 against 6.45 ms.)
+bool probe_attached();  // per-kernel timing: its events stand between the launches
+template <class... P, class... A>
+inline void launch_dependent(bool early, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                             A... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = early && !probe_attached() ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dependency_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+#endif
+
 // A cluster whose reduced system is solved in global memory (more than
 // kMaxFreeSmall free images): what the host needs to emit its launches.
 struct BigRef {
@@ -286,6 +316,8 @@ struct BigRef {
   std::vector<int> below;  // per block column of kBigNB: row blocks below it inside the envelope
   bool tc = true;          // tensor-core double-float factor (else the binary64 CUDA-core one)
   int panel_w = 4;         // column-block width of the panel factorisation (1, 2, 4, 8, 16 or 32)
+  bool early = false;      // its kernels by programmatic dependent launch: a single chain of launches, which has
+                           // the GPU to itself (beside others, CTAs that only wait would hold their SMs)
 };
 void launch_big_solve(const BigRef& b, bool mixed, int refine_steps, int assemble_only, cudaStream_t st);
 // rows of the digit buffer of a system of order n: n rounded up to kBigNB, plus
@@ -341,5 +373,19 @@ void launch_factor(const BatchView& bv, bool mixed, int refine_steps, int assemb
 void launch_fma_probe(int ctas, int iters, float* sink, cudaStream_t st);
 int chunk_obs(bool mixed);
 int chunk_tiles(bool mixed);
+// Tiles of a cluster's chunks when the launch parameters leave them open: the
+// precision's maximum, but for a small cluster fewer, so that its chunks cover
+// the SMs (152 of them in binary64, whose chunks are bound by the binary64
+// pipe of the SM they run on; half as many in mixed precision, whose chunks
+// are twice as large).  A cluster of 222 tiles in binary64 takes 70 us per
+// iteration in chunks of 8, 32 in chunks of 2.  Clusters of more than
+// kMaxFreeSmall free images, whose iteration is the global-memory solver's,
+// keep the maximum: their chunks hold more image pairs the smaller they are.
+inline int default_chunk_tiles(int n_tiles, int n_free, bool mixed) {
+  int t = n_free > kMaxFreeSmall ? kChunkTilesF64 : (n_tiles + 151) / 152;
+  t = t < 2 ? 2 : (t > kChunkTilesF64 ? kChunkTilesF64 : t);
+  return mixed ? 2 * t : t;
+}
+static_assert(kChunkTilesMixed == 2 * kChunkTilesF64, "chunk sizes of the two precisions");
 
 }  // namespace bagpu

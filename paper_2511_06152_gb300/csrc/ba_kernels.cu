@@ -1045,9 +1045,12 @@ __global__ void __launch_bounds__(kCostInitThreads) k_backsub_cost(BatchView bv)
   if (threadIdx.x == 0) n_due = 0;
   __syncthreads();
   const int lane = threadIdx.x & 31;
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int nwarps = (gridDim.x * blockDim.x) >> 5;
   const int total = bv.tot[0];
+  // few tiles: neighbouring ones go to different CTAs (a CTA of eight tiles
+  // would queue on the binary64 pipe of one SM while others have none)
+  const int warp = 2 * total <= nwarps ? (threadIdx.x >> 5) * gridDim.x + blockIdx.x
+                                       : (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   // each warp takes a contiguous run of tiles, so that its tiles mostly
   // belong to one cluster: it counts them per cluster and publishes the
   // count once per cluster it leaves (one fence and one atomic each); the
@@ -1222,7 +1225,7 @@ __device__ void backsub_tile(const DevCluster& C, LmState* lm, int local, int la
 template <bool MIXED>
 __global__ void __launch_bounds__(256) k_cost_tiles(BatchView bv) {
   const int lane = threadIdx.x & 31;
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int warp = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;  // few tiles spread over the SMs
   const int nwarps = (gridDim.x * blockDim.x) >> 5;
   const int total = bv.tot[0];
   for (int g = warp; g < total; g += nwarps) {
@@ -1606,6 +1609,7 @@ static thread_local Probe* t_probe = nullptr;
 static thread_local unsigned long long t_direct = 0, t_captured = 0;
 
 void set_probe(Probe* p) { t_probe = p; }
+bool probe_attached() { return t_probe != nullptr; }
 unsigned long long take_direct_launches() {
   const unsigned long long v = t_direct;
   t_direct = 0;
@@ -1693,10 +1697,16 @@ void launch_gather(const BatchView& bv, int iters, LmState* lm_out, StepRec* tra
   LAUNCH(KK_OTHER, st, k_gather<<<bv.n < 65535 ? bv.n : 65535, 128, 0, st>>>(bv, iters, lm_out, trace_out));
 }
 
+// tiles a CTA of eight warps is launched for: in binary64 one where that leaves
+// at most eight CTAs per SM (6 images: back-substitution 29 -> 22 us; in mixed
+// precision, not bound by a pipe of the SM, 12 images took 958 instead of 908 us
+// per 10 iterations that way)
+static int tiles_per_cta(const BatchView& bv, bool mixed) { return !mixed && bv.total_tiles <= 8 * num_sms() ? 1 : 8; }
+
 template <bool MIXED>
 static void launch_cost_init_t(const BatchView& bv, cudaStream_t st) {
   const int sms = num_sms();
-  LAUNCH(KK_COST_TILES, st, k_cost_tiles<MIXED><<<grid_for(bv.total_tiles, 8, sms * 16), 256, 0, st>>>(bv));
+  LAUNCH(KK_COST_TILES, st, k_cost_tiles<MIXED><<<grid_for(bv.total_tiles, tiles_per_cta(bv, MIXED), sms * 16), 256, 0, st>>>(bv));
   LAUNCH(KK_COST_INIT, st, k_cost_init<<<grid_for(bv.n, 1, 65535), kCostInitThreads, 0, st>>>(bv));
 }
 
@@ -1726,7 +1736,8 @@ static void launch_lin_schur(const BatchView& bv, int diag, cudaStream_t st) {
 template <bool MIXED>
 static void launch_partial_reduce(const BatchView& bv, int mirror, cudaStream_t st) {
   using Real = typename RealOf<MIXED>::T;
-  LAUNCH(KK_PARTIAL_REDUCE, st, k_partial_reduce<Real><<<grid_for(bv.total_items, 1, num_sms() * kRedCtasPerSm), kRedThreads, 0, st>>>(bv, mirror));
+  LAUNCH(KK_PARTIAL_REDUCE, st,
+         k_partial_reduce<Real><<<grid_for(bv.total_items, 1, num_sms() * kRedCtasPerSm), kRedThreads, 0, st>>>(bv, mirror));
 }
 
 template <bool MIXED>
@@ -1737,7 +1748,9 @@ static void launch_iteration_t(const BatchView& bv, int refine_steps, cudaStream
   launch_factor(bv, MIXED, refine_steps, 0, st);
   if (big)
     for (const BigRef& b : *big) launch_big_solve(b, MIXED, refine_steps, 0, st);
-  LAUNCH(KK_BACKSUB, st, k_backsub_cost<MIXED><<<grid_for(bv.total_tiles, 8, sms * bv.back_ctas_per_sm), kCostInitThreads, 0, st>>>(bv));
+  LAUNCH(KK_BACKSUB, st,
+         k_backsub_cost<MIXED><<<grid_for(bv.total_tiles, tiles_per_cta(bv, MIXED), sms * bv.back_ctas_per_sm),
+                                 kCostInitThreads, 0, st>>>(bv));
 }
 
 void launch_iteration(const BatchView& bv, bool mixed, int refine_steps, cudaStream_t st,
