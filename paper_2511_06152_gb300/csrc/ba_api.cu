@@ -446,8 +446,7 @@ ba_status get_plan(ba_ctx* ctx, const std::vector<ba_cluster_id>& ids, Plan** ou
   Plan* p = new Plan();
   p->ids = ids;
   auto big_ref = [&](const Cluster* c) {
-    return BigRef{c->d_desc, 6 * c->nf, c->nf, c->h.n_pairs, c->h.S, c->h.F, c->big_below, !ctx->big_fp64,
-                  ctx->tune.big_panel_w};
+    return BigRef{c->d_desc, 6 * c->nf, c->nf, c->h.n_pairs, c->h.S, c->h.F, c->big_below, !ctx->big_fp64};
   };
   for (int i = 0; i < n; ++i) {
     Cluster* c = find_cluster(ctx, ids[i]);
@@ -3052,7 +3051,6 @@ BA_API ba_status ba_autotune(ba_ctx* ctx, const ba_cluster_desc* descs, int32_t 
   if (!ctx || !descs || n <= 0 || iters <= 0 || !out) return BA_ERR_INVALID;
   std::vector<ba_cluster_id> ids;
   int created = -1;  // chunk_tiles the current tuning clusters were created with
-  bool has_big = false;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   auto destroy_all = [&]() {
     for (ba_cluster_id id : ids) ba_destroy_cluster(ctx, id);
@@ -3080,8 +3078,6 @@ BA_API ba_status ba_autotune(ba_ctx* ctx, const ba_cluster_desc* descs, int32_t 
         st = ba_create_cluster(ctx, &descs[i], &id);
         if (st != BA_OK) return st;
         ids.push_back(id);
-        ba_cluster_info info{};
-        if (ba_get_cluster_info(ctx, id, &info) == BA_OK && info.n_free > kMaxFreeSmall) has_big = true;
       }
       created = ct;
     }
@@ -3112,19 +3108,16 @@ BA_API ba_status ba_autotune(ba_ctx* ctx, const ba_cluster_desc* descs, int32_t 
   struct Knob {
     int TuneParams::*field;
     std::vector<int> cands;
-    bool big_only;
   };
   const bool mixed = ctx->mixed;
   const std::vector<Knob> knobs = {
-      {&TuneParams::chunk_tiles, mixed ? std::vector<int>{12, 8} : std::vector<int>{6, 4}, false},
-      {&TuneParams::lin_ctas_per_sm, {4, 2}, false},
-      {&TuneParams::back_ctas_per_sm, {8, 4}, false},
-      {&TuneParams::factor_threads, {384, 256}, false},
-      {&TuneParams::big_panel_w, {2, 8}, true},
-      {&TuneParams::batch_chains, {2, 8}, false},
+      {&TuneParams::chunk_tiles, mixed ? std::vector<int>{12, 8} : std::vector<int>{6, 4}},
+      {&TuneParams::lin_ctas_per_sm, {4, 2}},
+      {&TuneParams::back_ctas_per_sm, {8, 4}},
+      {&TuneParams::factor_threads, {384, 256}},
+      {&TuneParams::batch_chains, {2, 8}},
   };
   for (const Knob& k : knobs) {
-    if (k.big_only && !has_big) continue;
     TuneParams best = cur;
     double best_ms = cur_ms;
     for (int v : k.cands) {

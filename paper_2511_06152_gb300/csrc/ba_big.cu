@@ -15,7 +15,7 @@
 //   k_big_split      S -> F (lower triangle, double-float, zeros outside the envelope)
 //   per block column k of kBigNB columns (right-looking):
 //     k_big_panel      every CTA factors the diagonal block and inverts it
-//                      (double-float); CTA 0 stores both, CTA b stores the
+//                      (double-float); CTA 0 stores the inverse, CTA b the
 //                      panel L_ik = A_ik L_kk^-T of row block k + b and its
 //                      Ozaki digits
 //     k_big_update_tc  A_ij -= L_ik L_jk^T on 128 x 32 tiles inside the
@@ -43,6 +43,7 @@
 
 #include <algorithm>
 
+#include "ba_block.cuh"
 #include "ba_camera.cuh"
 #include "ba_device.cuh"
 #include "ba_internal.h"
@@ -407,143 +408,109 @@ constexpr int kPld = kBigNB + 1;  // padded leading dimension of the shared bloc
 
 // Block column k: the diagonal block factored and inverted by every CTA
 // (double-float; rows past n padded with the identity), then CTA 0 stores
-// the factor and the inverse, CTA b (1 <= b <= m) the panel of row block
-// k + b, L_ik = A_ik (L_kk^-1)^T, and its Ozaki digits and row scales.
+// the inverse, CTA b (1 <= b <= m) the panel of row block k + b,
+// L_ik = A_ik (L_kk^-1)^T, and its Ozaki digits and row scales.
 //
-// The factor and its inverse come out of one right-looking sweep: W starts
-// as the identity and receives the same row operations as the matrix, so
-// that row j of W, scaled by 1 / L(j, j) once the column j is final, is row
-// j of L^-1 (forward substitution of L X = I, one row at a time).  Columns
-// go in blocks of pw (a divisor of 32): one warp factors a block (the
-// pivots' reciprocal square roots, the block's columns of L, its rows of X)
-// with warp-level synchronisation only, then the whole CTA applies the
-// block's rank-pw update below it: two block-wide barriers per block.
-__global__ void __launch_bounds__(kPanelThreads) k_big_panel(const DevCluster* dcl, int k, int pw) {
+// The 32 x 32 block goes as 4 x 4 blocks of 8 (ba_block.cuh), L D L^T with the
+// identity as 32 more rows below it: the same sweeps turn those into the
+// columns of the unit factor's inverse.  Per block column of 8: two warps sweep
+// its eight pivots with three row blocks each, then a warp per block applies
+// the products to what is right of it; two barriers.  (The predecessor, a
+// column at a time with rank-pw updates by the whole CTA, took 22 k cycles of
+// the launch's 56 k; a sweep takes 1.2 k.)
+__global__ void __launch_bounds__(kPanelThreads) k_big_panel(const DevCluster* dcl, int k) {
   dependency_wait();
   dependency_trigger();
   const DevCluster& C = *dcl;
   const int n = 6 * C.n_free, r0 = kBigNB * k, nb = min(kBigNB, n - r0);
   float* Fh = df_hi(C);
   float* Fl = df_lo(C);
-  __shared__ float Lh[kBigNB][kPld], Ll[kBigNB][kPld];  // factor
-  __shared__ float Wh[kBigNB][kPld], Wl[kBigNB][kPld];  // identity -> inverse of the factor
-  __shared__ float Ph[kBigNB][kPld], Pl[kBigNB][kPld];  // A_ik
-  const int tid = threadIdx.x;
+  constexpr int kB = kBigNB / 8;  // 8 x 8 blocks along the diagonal block
+  // blocks (i, j): rows 0 .. kB - 1 the matrix, kB .. 2 kB - 1 the identity
+  __shared__ __align__(16) char blocks[2 * kB * kB * kBlkBytes];
+  __shared__ __align__(16) char ybuf[kB * kBlkBytes];            // y of the matrix's row blocks, current column
+  __shared__ dfl sq[kBigNB];                                      // sqrt(d)
+  __shared__ float Wh[kBigNB][kPld], Wl[kBigNB][kPld];           // inverse of the factor
+  __shared__ float Ph[kBigNB][kPld], Pl[kBigNB][kPld];           // A_ik
+  __shared__ int s_fail;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int b = blockIdx.x;
   const int ri = r0 + kBigNB * b, nr = b == 0 ? nb : min(kBigNB, n - ri);
-  for (int idx = tid; idx < kBigNB * kBigNB; idx += kPanelThreads) {
-    const int r = idx >> 5, c = idx & 31;
-    float h = 0.0f, l = 0.0f;
+  auto blk = [&](int i, int j) { return blocks + (i * kB + j) * kBlkBytes; };
+  if (tid == 0) s_fail = 0;
+  {
+    const int r = tid >> 5, c = tid & 31;  // kPanelThreads = 32 x 32
+    dfl v{0.0f, 0.0f};
     if (r < nb && c < nb) {
-      if (c <= r) {
-        h = Fh[(size_t)(r0 + r) * n + r0 + c];
-        l = Fl[(size_t)(r0 + r) * n + r0 + c];
-      }
+      if (c <= r) v = dfl{Fh[(size_t)(r0 + r) * n + r0 + c], Fl[(size_t)(r0 + r) * n + r0 + c]};
     } else if (r == c) {
-      h = 1.0f;
+      v.hi = 1.0f;
     }
-    Lh[r][c] = h;
-    Ll[r][c] = l;
-    Wh[r][c] = r == c ? 1.0f : 0.0f;
-    Wl[r][c] = 0.0f;
+    *reinterpret_cast<dfl*>(blk(r >> 3, c >> 3) + elt_off(r & 7, c & 7)) = v;
+    *reinterpret_cast<dfl*>(blk(kB + (r >> 3), c >> 3) + elt_off(r & 7, c & 7)) = dfl{r == c ? 1.0f : 0.0f, 0.0f};
     if (b > 0) {
-      float ph = 0.0f, pl = 0.0f;
-      if (r < nr && c < nb) {
-        ph = Fh[(size_t)(ri + r) * n + r0 + c];
-        pl = Fl[(size_t)(ri + r) * n + r0 + c];
-      }
-      Ph[r][c] = ph;
-      Pl[r][c] = pl;
+      dfl p{0.0f, 0.0f};
+      if (r < nr && c < nb) p = dfl{Fh[(size_t)(ri + r) * n + r0 + c], Fl[(size_t)(ri + r) * n + r0 + c]};
+      Ph[r][c] = p.hi;
+      Pl[r][c] = p.lo;
     }
   }
-  __shared__ float Dh[kBigNB], Dl[kBigNB];  // L(j, j), kept apart until the sweep ends
   __syncthreads();
-  bool fail = false;
-  // blocks of pw columns: warp 0 factors the block's columns (lane = row,
-  // warp-level synchronisation only) and finishes the block's rows of X;
-  // then every thread applies the block's rank-pw update to the rows below
-  // it (entry (tr, tc) of the trailing matrix, or of W left of it)
-  const int tr = tid >> 5, tc = tid & 31, lane = tid & 31;
-  for (int jb = 0; jb < kBigNB; jb += pw) {
-    const int je = jb + pw - 1;  // last column of the block
-    if (tid < 32) {
-      for (int j = jb; j <= je; ++j) {
-        dfl d{Lh[j][j], Ll[j][j]};
-        if (!(d.hi > 0.0f)) {
-          fail = true;
-          d = dfl{1.0f, 0.0f};
-        }
-        const dfl iv = df_rsqrt(d);
-        if (lane > j) {
-          const dfl v = df_mul(dfl{Lh[lane][j], Ll[lane][j]}, iv);
-          Lh[lane][j] = v.hi;
-          Ll[lane][j] = v.lo;
+  for (int p = 0; p < kB; ++p) {
+    // the row blocks below the pivots: the matrix's p + 1 .. kB - 1, the
+    // identity's 0 .. p (the later ones are still zero in this column)
+    if (warp < 2) {
+      const int q = lane >> 3, t = 3 * warp + q - 1, row = lane & 7;
+      const bool has = q > 0 && t < kB;
+      const int i = has ? (t < kB - 1 - p ? p + 1 + t : kB + t - (kB - 1 - p)) : p;
+      dfl a[8], l[8], r{1.0f, 0.0f};
+      float s = 1.0f;
+      ld_row<dfl>(blk(i, p), row, a);
+      if (!sweep_warp<ArithDf>(a, l, r, s, lane) && lane == 0) s_fail = 1;
+      __syncwarp();
+      if (has) {
+        st_row<dfl>(blk(i, p), row, l);
+        if (i < kB) st_row<dfl>(ybuf + i * kBlkBytes, row, a);
+      } else if (warp == 0 && q == 0) {
+        const dfl e = df_rsqrt(r);  // sqrt(d s)
+        const float h = s == 1.0f ? 1.0f : 0x1p-50f;
+        sq[8 * p + row] = dfl{e.hi * h, e.lo * h};
+      }
+    }
+    __syncthreads();
+    if (p + 1 < kB) {
+      // blocks (i, j), j > p: the matrix's i = j .. kB - 1, the identity's 0 .. p
+      const int m = kB - 1 - p, na = m * (m + 1) / 2;
+      for (int t = warp; t < na + (p + 1) * m; t += kPanelThreads / 32) {
+        int i, j;
+        if (t < na) {
+          int u = t;
+          for (j = p + 1; u >= kB - j; ++j) u -= kB - j;
+          i = j + u;
         } else {
-          if (lane == j) {
-            const dfl sq = df_mul(d, iv);
-            Dh[j] = sq.hi;
-            Dl[j] = sq.lo;
-          }
-          const dfl x = df_mul(dfl{Wh[j][lane], Wl[j][lane]}, iv);  // row j of X
-          Wh[j][lane] = x.hi;
-          Wl[j][lane] = x.lo;
+          i = kB + (t - na) / m;
+          j = p + 1 + (t - na) % m;
         }
-        __syncwarp();
-        if (lane > j) {  // the block's later columns, rows below j
-          const dfl lr{Lh[lane][j], Ll[lane][j]};
-          for (int c = j + 1; c <= je && c <= lane; ++c) {
-            const dfl a = df_fms(dfl{Lh[lane][c], Ll[lane][c]}, lr, dfl{Lh[c][j], Ll[c][j]});
-            Lh[lane][c] = a.hi;
-            Ll[lane][c] = a.lo;
-          }
-        }
-        if (lane <= j) {  // the block's later rows of W, column lane
-          const dfl xj{Wh[j][lane], Wl[j][lane]};
-          for (int r = j + 1; r <= je; ++r) {
-            const dfl a = df_fms(dfl{Wh[r][lane], Wl[r][lane]}, dfl{Lh[r][j], Ll[r][j]}, xj);
-            Wh[r][lane] = a.hi;
-            Wl[r][lane] = a.lo;
-          }
-        }
-        __syncwarp();
+        product_warp<ArithDf>(blk(i, j), blk(i, p), ybuf + j * kBlkBytes, lane);
       }
+      __syncthreads();
     }
-    __syncthreads();
-    if (tr > je && tc <= tr) {
-      if (tc <= je) {  // W(tr, tc) -= sum_j L(tr, j) X(j, tc) over the block's columns
-        dfl a{Wh[tr][tc], Wl[tr][tc]};
-        for (int i = 0; i < pw; ++i) {
-          const int j = jb + i;
-          if (j >= tc) a = df_fms(a, dfl{Lh[tr][j], Ll[tr][j]}, dfl{Wh[j][tc], Wl[j][tc]});
-        }
-        Wh[tr][tc] = a.hi;
-        Wl[tr][tc] = a.lo;
-      } else {  // L(tr, tc) -= sum_j L(tr, j) L(tc, j)
-        dfl a{Lh[tr][tc], Ll[tr][tc]};
-        for (int i = 0; i < pw; ++i) a = df_fms(a, dfl{Lh[tr][jb + i], Ll[tr][jb + i]}, dfl{Lh[tc][jb + i], Ll[tc][jb + i]});
-        Lh[tr][tc] = a.hi;
-        Ll[tr][tc] = a.lo;
-      }
-    }
-    __syncthreads();
   }
-  if (tid < kBigNB) {
-    Lh[tid][tid] = Dh[tid];
-    Ll[tid][tid] = Dl[tid];
+  {  // inverse(r, c) = sqrt(d_r) l_c(r), r >= c
+    const int r = tid >> 5, c = tid & 31;
+    dfl v{0.0f, 0.0f};
+    if (c <= r)
+      v = df_mul(*reinterpret_cast<const dfl*>(blk(kB + (c >> 3), r >> 3) + elt_off(c & 7, r & 7)), sq[r]);
+    Wh[r][c] = v.hi;
+    Wl[r][c] = v.lo;
   }
   __syncthreads();
   if (b == 0) {
-    if (tid == 0 && fail) *C.bflag = 1;
+    if (tid == 0 && s_fail) *C.bflag = 1;
     float* lv = C.linv + (size_t)k * 2 * kBigNB * kBigNB;
-    for (int idx = tid; idx < kBigNB * kBigNB; idx += kPanelThreads) {
-      const int r = idx >> 5, c = idx & 31;
-      lv[idx] = Wh[r][c];
-      lv[kBigNB * kBigNB + idx] = Wl[r][c];
-      if (r < nb && c <= r) {
-        Fh[(size_t)(r0 + r) * n + r0 + c] = Lh[r][c];
-        Fl[(size_t)(r0 + r) * n + r0 + c] = Ll[r][c];
-      }
-    }
+    const int r = tid >> 5, c = tid & 31;
+    lv[tid] = Wh[r][c];
+    lv[kBigNB * kBigNB + tid] = Wl[r][c];
     return;
   }
   // the panel: L_ik(r, c) = sum_{q <= c} A_ik(r, q) X(c, q), thread (r, c)
@@ -843,7 +810,7 @@ void launch_big_solve(const BigRef& b, bool mixed, int refine_steps, int assembl
     LAUNCH(KK_FACTOR, st, launch_dependent(b.early, k_big_split, std::min(n, num_sms() * 8), 256, 0, st, b.d));
     for (int k = 0; k < nblk; ++k) {
       const int m = b.below[k];
-      LAUNCH(KK_FACTOR, st, launch_dependent(b.early, k_big_panel, 1 + m, kPanelThreads, 0, st, b.d, k, b.panel_w));
+      LAUNCH(KK_FACTOR, st, launch_dependent(b.early, k_big_panel, 1 + m, kPanelThreads, 0, st, b.d, k));
       if (m > 0) {
         const dim3 grid(m, (kBigNB * m + kUpdM - 1) / kUpdM);
         LAUNCH(KK_FACTOR, st, launch_dependent(b.early, k_big_update_tc, grid, kUpdThreads, kUpdSmem, st, b.d, k, m));

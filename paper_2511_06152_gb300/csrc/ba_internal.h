@@ -224,7 +224,7 @@ struct TuneParams {
   int back_ctas_per_sm = 16;
   int factor_nb = 8;         // kept for its place in the interface: the factor's block columns are 8 wide
   int factor_threads = 512;
-  int big_panel_w = 4;       // columns of a block of the global-memory solver's panel factorisation
+  int big_panel_w = 4;       // kept for its place in the interface: the panels' blocks are 8 wide
   int batch_chains = 4;      // concurrent launch chains of a batch's LM iterations
 };
 
@@ -315,7 +315,6 @@ struct BigRef {
   double* F;               // device [n][n]
   std::vector<int> below;  // per block column of kBigNB: row blocks below it inside the envelope
   bool tc = true;          // tensor-core double-float factor (else the binary64 CUDA-core one)
-  int panel_w = 4;         // column-block width of the panel factorisation (1, 2, 4, 8, 16 or 32)
   bool early = false;      // its kernels by programmatic dependent launch: a single chain of launches, which has
                            // the GPU to itself (beside others, CTAs that only wait would hold their SMs)
 };
