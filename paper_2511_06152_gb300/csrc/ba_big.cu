@@ -17,13 +17,16 @@
 //     k_big_panel      every CTA factors the diagonal block and inverts it
 //                      (double-float); CTA 0 stores the inverse, CTA b the
 //                      panel L_ik = A_ik L_kk^-T of row block k + b and its
-//                      Ozaki digits
+//                      Ozaki digits; forward substitution of the block column
 //     k_big_update_tc  A_ij -= L_ik L_jk^T on 128 x 32 tiles inside the
 //                      envelope: digit products on the tensor cores,
 //                      double-float subtraction
-//   k_big_solve_df   forward and backward substitution (one CTA, double-float,
+//   k_big_back       backward substitution (a cluster of 8 CTAs, double-float,
 //                    the inverted diagonal blocks and the panels)
-//   k_big_resid      t = rhs - S x in binary64
+//   per refinement step:
+//     k_big_resid      t = rhs - S x in binary64
+//     k_big_forward    forward substitution of t (one CTA)
+//     k_big_back       x += its backward substitution
 //   k_big_finish     the images' steps, candidate poses, pred and prior terms, status
 //
 // Binary64 factorisation on the CUDA cores (BA_FLAG_BIG_FP64_FACTOR):
@@ -39,6 +42,7 @@
 // ef(r) = 6 env_first[r / 6]; the rows of a column block that can be nonzero
 // below it form one contiguous run of row blocks, whose length per block
 // column the host passes in (it fixes the grid sizes).
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -381,6 +385,22 @@ __device__ __forceinline__ float* df_lo(const DevCluster& C) {
 
 // F = S on the lower triangle as double-float (entries outside the envelope
 // are zero in S and become zero here), one CTA per row.
+// The forward substitution's vectors on the tensor-core path, n double-floats
+// each in bx: v (the right-hand side less what the block columns done so far
+// take off it) and y = L^-1 rhs.
+__device__ __forceinline__ dfl* fwd_v(const DevCluster& C) { return reinterpret_cast<dfl*>(C.bx); }
+__device__ __forceinline__ dfl* fwd_y(const DevCluster& C) {
+  return reinterpret_cast<dfl*>(C.bx + 3 * (size_t)(6 * C.n_free));
+}
+
+// Dot2 partial sums of a warp (or of aligned groups of `width` lanes)
+// merged by a butterfly: every lane ends with the group's total.
+__device__ __forceinline__ Dot2 warp_merge(Dot2 d, int width) {
+  for (int off = 1; off < width; off <<= 1)
+    d.merge(__shfl_xor_sync(BA_FULL_MASK, d.s, off), __shfl_xor_sync(BA_FULL_MASK, d.c, off));
+  return d;
+}
+
 __global__ void __launch_bounds__(256) k_big_split(const DevCluster* dcl) {
   dependency_wait();
   dependency_trigger();
@@ -388,6 +408,8 @@ __global__ void __launch_bounds__(256) k_big_split(const DevCluster* dcl) {
   const int n = 6 * C.n_free;
   float* Fh = df_hi(C);
   float* Fl = df_lo(C);
+  dfl* v = fwd_v(C);
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) v[i] = df_from_d(C.rhs[i]);
   for (int r = blockIdx.x; r < n; r += gridDim.x) {
     const double* srow = C.S + (size_t)r * n;
     for (int c = threadIdx.x; c <= r; c += blockDim.x) {
@@ -418,6 +440,11 @@ constexpr int kPld = kBigNB + 1;  // padded leading dimension of the shared bloc
 // the products to what is right of it; two barriers.  (The predecessor, a
 // column at a time with rank-pw updates by the whole CTA, took 22 k cycles of
 // the launch's 56 k; a sweep takes 1.2 k.)
+//
+// The right-hand side goes along as one more row of the matrix: every CTA takes
+// y_k = L_kk^-1 v_k, CTA 0 stores it and CTA b subtracts L_ik y_k from v_i: a
+// warp sum per row here, against a sweep over the whole factor of its own in one
+// CTA (with the backward one, 663 us at n = 2400).
 __global__ void __launch_bounds__(kPanelThreads) k_big_panel(const DevCluster* dcl, int k) {
   dependency_wait();
   dependency_trigger();
@@ -432,6 +459,7 @@ __global__ void __launch_bounds__(kPanelThreads) k_big_panel(const DevCluster* d
   __shared__ dfl sq[kBigNB];                                      // sqrt(d)
   __shared__ float Wh[kBigNB][kPld], Wl[kBigNB][kPld];           // inverse of the factor
   __shared__ float Ph[kBigNB][kPld], Pl[kBigNB][kPld];           // A_ik
+  __shared__ dfl vk[kBigNB], yk[kBigNB];                          // the right-hand side's part
   __shared__ int s_fail;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int b = blockIdx.x;
@@ -454,6 +482,7 @@ __global__ void __launch_bounds__(kPanelThreads) k_big_panel(const DevCluster* d
       Ph[r][c] = p.hi;
       Pl[r][c] = p.lo;
     }
+    if (tid < kBigNB) vk[tid] = tid < nb ? fwd_v(C)[r0 + tid] : dfl{0.0f, 0.0f};
   }
   __syncthreads();
   for (int p = 0; p < kB; ++p) {
@@ -505,7 +534,15 @@ __global__ void __launch_bounds__(kPanelThreads) k_big_panel(const DevCluster* d
     Wl[r][c] = v.lo;
   }
   __syncthreads();
+  {  // y_k(r) = sum_q X(r, q) v_k(q): a warp per row
+    Dot2 acc;
+    if (lane <= warp) acc.add(dfl{Wh[warp][lane], Wl[warp][lane]}, vk[lane]);
+    acc = warp_merge(acc, 32);
+    if (lane == 0) yk[warp] = acc.get();
+  }
   if (b == 0) {
+    __syncthreads();
+    if (tid < nb) fwd_y(C)[r0 + tid] = yk[tid];
     if (tid == 0 && s_fail) *C.bflag = 1;
     float* lv = C.linv + (size_t)k * 2 * kBigNB * kBigNB;
     const int r = tid >> 5, c = tid & 31;
@@ -534,6 +571,14 @@ __global__ void __launch_bounds__(kPanelThreads) k_big_panel(const DevCluster* d
 #pragma unroll
   for (int t = 0; t < kSlices; ++t) C.dig[(size_t)t * slice + off] = dg[t];
   if (c == 0) C.dexp[row] = E;
+  __syncthreads();  // yk
+  Dot2 dv;          // v_i(r) -= sum_c L_ik(r, c) y_k(c)
+  if (live) dv.add(out, yk[c]);
+  dv = warp_merge(dv, 32);
+  if (c == 0 && r < nr) {
+    dfl* v = fwd_v(C) + row;
+    *v = df_sub(*v, dv.get());
+  }
 }
 
 constexpr int kUpdThreads = 512;  // 16 warps: 4 per tensor-memory lane quarter, 8 columns each
@@ -650,29 +695,19 @@ __global__ void __launch_bounds__(kUpdThreads, 1) k_big_update_tc(const DevClust
   if (warp == 0) tmem_dealloc(tmem, kUpdTmemCols);
 }
 
-// Dot2 partial sums of a warp (or of aligned groups of `width` lanes)
-// merged by a butterfly: every lane ends with the group's total.
-__device__ __forceinline__ Dot2 warp_merge(Dot2 d, int width) {
-  for (int off = 1; off < width; off <<= 1)
-    d.merge(__shfl_xor_sync(BA_FULL_MASK, d.s, off), __shfl_xor_sync(BA_FULL_MASK, d.c, off));
-  return d;
-}
-
 size_t big_solve_df_smem(int n) { return sizeof(float) * (2 * (size_t)n + 2 * kBigNB); }
 
 constexpr int kSolveChunk = 12;  // entries a lane loads before it sums them
 
-// Solve S y = v with the double-float factor (one CTA of 1024 threads; v in
-// shared memory).  Both sweeps read, per block k of 32 rows, the rows' own
-// entries left of the diagonal block, L(r0 + r, lo .. r0), lo = the block's
-// first envelope column (contiguous in memory: coalesced across a warp), and
-// the inverted diagonal block X = L_kk^-1 (loaded one block ahead).
-//   forward  (k ascending):  u = v_k - L(k, lo .. r0) v(lo .. r0); v_k = X u
-//   backward (k descending): x_k = X^T v_k; v(lo .. r0) -= L(k, lo .. r0)^T x_k
+// Forward substitution y = L^-1 t of a refinement step's residual (one CTA of
+// 1024 threads; the vector in shared memory).  Per block k of 32 rows it reads
+// the rows' own entries left of the diagonal block, L(r0 + r, lo .. r0), lo =
+// the block's first envelope column (contiguous in memory: coalesced across a
+// warp), and the inverted diagonal block X = L_kk^-1:
+//   u = v_k - L(k, lo .. r0) v(lo .. r0);  y_k = X u
 // Every dot product is compensated (Dot2); each lane issues its loads in
-// groups of kSolveChunk before it sums them.  x = S^-1 rhs (mode 0) or
-// x += S^-1 t (mode 1), binary64 in and out.
-__global__ void __launch_bounds__(1024) k_big_solve_df(const DevCluster* dcl, int mode) {
+// groups of kSolveChunk before it sums them.
+__global__ void __launch_bounds__(1024) k_big_forward(const DevCluster* dcl) {
   dependency_wait();
   dependency_trigger();
   const DevCluster& C = *dcl;
@@ -684,7 +719,7 @@ __global__ void __launch_bounds__(1024) k_big_solve_df(const DevCluster* dcl, in
   float* yl = yh + kBigNB;
   const float* Fh = df_hi(C);
   const float* Fl = df_lo(C);
-  const double* src = mode == 0 ? C.rhs : C.bx + 2 * n;
+  const double* src = C.bx + 2 * n;
   for (int i = tid; i < n; i += blockDim.x) {
     const dfl v = df_from_d(src[i]);
     vh[i] = v.hi;
@@ -692,7 +727,7 @@ __global__ void __launch_bounds__(1024) k_big_solve_df(const DevCluster* dcl, in
   }
   const int nblk = (n + kBigNB - 1) / kBigNB;
   const size_t xs = 2 * kBigNB * kBigNB;
-  // this thread's entry of X: (wid, lane) in the forward sweep, (lane, wid) in the backward one
+  // this thread's entry of X, (wid, lane), one block ahead
   float xh = C.linv[wid * kBigNB + lane], xl = C.linv[kBigNB * kBigNB + wid * kBigNB + lane];
   __syncthreads();
   for (int k = 0; k < nblk; ++k) {  // L y = v
@@ -739,53 +774,97 @@ __global__ void __launch_bounds__(1024) k_big_solve_df(const DevCluster* dcl, in
     }
     __syncthreads();
   }
-  xh = C.linv[(nblk - 1) * xs + lane * kBigNB + wid];
-  xl = C.linv[(nblk - 1) * xs + kBigNB * kBigNB + lane * kBigNB + wid];
-  for (int k = nblk - 1; k >= 0; --k) {  // L^T x = y
-    const int r0 = kBigNB * k, nb = min(kBigNB, n - r0), lo = ef_row(C, r0);
-    {  // warp r: x_r = sum_q X(q, r) y_q
-      Dot2 acc;
-      if (lane < nb) acc.add(dfl{xh, xl}, dfl{vh[r0 + lane], vl[r0 + lane]});
-      acc = warp_merge(acc, 32);
-      if (lane == 0) {
-        const dfl x = acc.get();
-        yh[wid] = x.hi;
-        yl[wid] = x.lo;
-      }
-    }
-    if (k > 0) {
-      xh = C.linv[(k - 1) * xs + lane * kBigNB + wid];
-      xl = C.linv[(k - 1) * xs + kBigNB * kBigNB + lane * kBigNB + wid];
-    }
-    __syncthreads();
-    if (tid < nb) {
-      vh[r0 + tid] = yh[tid];
-      vl[r0 + tid] = yl[tid];
-    }
-    for (int j = lo + tid; j < r0; j += blockDim.x) {  // v_j -= sum_r L(r0 + r, j) x_r
-      Dot2 acc;
-      for (int q0 = 0; q0 < nb; q0 += kSolveChunk) {
-        float ah[kSolveChunk], al[kSolveChunk];
-#pragma unroll
-        for (int i = 0; i < kSolveChunk; ++i) {
-          const size_t o = (size_t)(r0 + q0 + i) * n + j;
-          ah[i] = q0 + i < nb ? Fh[o] : 0.0f;
-          al[i] = q0 + i < nb ? Fl[o] : 0.0f;
-        }
-#pragma unroll
-        for (int i = 0; i < kSolveChunk; ++i)
-          if (q0 + i < nb) acc.add(dfl{ah[i], al[i]}, dfl{yh[q0 + i], yl[q0 + i]});
-      }
-      const dfl v = df_sub(dfl{vh[j], vl[j]}, acc.get());
-      vh[j] = v.hi;
-      vl[j] = v.lo;
-    }
-    __syncthreads();
-  }
+  for (int i = tid; i < n; i += blockDim.x) fwd_y(C)[i] = dfl{vh[i], vl[i]};
+}
+
+// Backward substitution x = L^-T y, k descending:
+//   x_k = X^T y_k;  y(lo .. r0) -= L(k, lo .. r0)^T x_k
+// A chain of block columns, bound by the latency of each step.  A cluster of
+// kBackCtas CTAs holds y, block column j in CTA j mod kBackCtas: that CTA forms
+// x_j (a warp per entry) and writes it into every CTA's buffer (two, in turn);
+// after the cluster's barrier each CTA updates its own columns, four lanes per
+// column with eight rows each, from entries of L loaded before the barrier.
+// x = (mode 0) or x += (mode 1) in binary64.  (400 images, n = 2400, three
+// iterations, with the forward sweep moved into the panels: 9.75 ms -> 8.98 ms;
+// 120 images 3.04 -> 2.94 ms.  The one CTA before it took about 4 us a step.)
+constexpr int kBackCtas = 8, kBackRows = kBigNB / 4;
+
+__global__ void __cluster_dims__(kBackCtas) __launch_bounds__(1024) k_big_back(const DevCluster* dcl, int mode) {
+  dependency_wait();
+  dependency_trigger();
+  const DevCluster& C = *dcl;
+  extern __shared__ dfl sy[];  // [n], its own block columns current
+  __shared__ dfl xbuf[2][kBigNB];
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = (int)cl.block_rank();
+  const int n = 6 * C.n_free, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int c8 = lane & 7, g = lane >> 3;  // column of the warp's eight, quarter of the rows
+  const float* Fh = df_hi(C);
+  const float* Fl = df_lo(C);
   double* x = C.bx + n;
-  for (int i = tid; i < n; i += blockDim.x) {
-    const double v = (double)vh[i] + (double)vl[i];
-    x[i] = mode == 0 ? v : x[i] + v;
+  for (int i = tid; i < n; i += blockDim.x) sy[i] = fwd_y(C)[i];
+  const int nblk = (n + kBigNB - 1) / kBigNB;
+  const size_t xs = 2 * kBigNB * kBigNB;
+  // entry (lane, wid) of X of the CTA's next block column
+  int own = nblk - 1 - ((nblk - 1 - rank) & (kBackCtas - 1));
+  float xh = 0.0f, xl = 0.0f;
+  if (own >= 0 && own < nblk) {
+    xh = C.linv[own * xs + lane * kBigNB + wid];
+    xl = C.linv[own * xs + kBigNB * kBigNB + lane * kBigNB + wid];
+  }
+  cl.sync();  // every CTA of the cluster runs before its buffer is written; sy
+  for (int k = nblk - 1; k >= 0; --k) {
+    const int r0 = kBigNB * k, nb = min(kBigNB, n - r0), lo = ef_row(C, r0);
+    // the CTA's block columns inside the envelope: j0, j0 + kBackCtas, .. < k; eight columns a warp
+    const int lb = lo / kBigNB, j0 = lb + ((rank - lb) & (kBackCtas - 1));
+    const int items = j0 < k ? 4 * ((k - 1 - j0) / kBackCtas + 1) : 0;
+    auto column = [&](int t) { return kBigNB * (j0 + kBackCtas * (t >> 2)) + 8 * (t & 3) + c8; };
+    float ah[kBackRows], al[kBackRows];
+    auto load = [&](int t) {
+      const int j = column(t);
+      const bool has = t < items && j >= lo;
+#pragma unroll
+      for (int i = 0; i < kBackRows; ++i) {
+        const int q = kBackRows * g + i;
+        const size_t o = (size_t)(r0 + q) * n + j;
+        ah[i] = has && q < nb ? Fh[o] : 0.0f;
+        al[i] = has && q < nb ? Fl[o] : 0.0f;
+      }
+    };
+    load(wid);
+    if (rank == (k & (kBackCtas - 1))) {  // warp r: x_r = sum_q X(q, r) y_q
+      Dot2 acc;
+      if (lane < nb) acc.add(dfl{xh, xl}, sy[r0 + lane]);
+      acc = warp_merge(acc, 32);
+      const dfl v = acc.get();
+      if (lane < kBackCtas) cl.map_shared_rank(&xbuf[k & 1][0], lane)[wid] = v;
+      if (lane == 0 && wid < nb) {
+        const double d = (double)v.hi + (double)v.lo;
+        x[r0 + wid] = mode == 0 ? d : x[r0 + wid] + d;
+      }
+      own -= kBackCtas;
+      if (own >= 0) {
+        xh = C.linv[own * xs + lane * kBigNB + wid];
+        xl = C.linv[own * xs + kBigNB * kBigNB + lane * kBigNB + wid];
+      }
+    }
+    cl.sync();
+    const dfl* xk = xbuf[k & 1];
+    for (int t = wid; t < items; t += 32) {  // y_j -= sum_r L(r0 + r, j) x_r
+      if (t != wid) load(t);
+      Dot2 acc;
+#pragma unroll
+      for (int i = 0; i < kBackRows; ++i) acc.add(dfl{ah[i], al[i]}, xk[kBackRows * g + i]);
+#pragma unroll
+      for (int off = 8; off < 32; off <<= 1)
+        acc.merge(__shfl_xor_sync(BA_FULL_MASK, acc.s, off), __shfl_xor_sync(BA_FULL_MASK, acc.c, off));
+      if (g == 0) {
+        const int j = column(t);
+        sy[j] = df_sub(sy[j], acc.get());
+      }
+    }
+    if (rank == ((k - 1) & (kBackCtas - 1))) __syncthreads();  // sy, for the next step's owner
   }
 }
 
@@ -817,10 +896,11 @@ void launch_big_solve(const BigRef& b, bool mixed, int refine_steps, int assembl
       }
     }
     const size_t sm = big_solve_df_smem(n);
-    LAUNCH(KK_FACTOR, st, launch_dependent(b.early, k_big_solve_df, 1, 1024, sm, st, b.d, 0));
+    LAUNCH(KK_FACTOR, st, launch_dependent(b.early, k_big_back, kBackCtas, 1024, sm, st, b.d, 0));
     for (int it = 0; it < refine_steps; ++it) {
       LAUNCH(KK_FACTOR, st, launch_dependent(b.early, k_big_resid, grid_for_big(n * 32, 256), 256, 0, st, b.d));
-      LAUNCH(KK_FACTOR, st, launch_dependent(b.early, k_big_solve_df, 1, 1024, sm, st, b.d, 1));
+      LAUNCH(KK_FACTOR, st, launch_dependent(b.early, k_big_forward, 1, 1024, sm, st, b.d));
+      LAUNCH(KK_FACTOR, st, launch_dependent(b.early, k_big_back, kBackCtas, 1024, sm, st, b.d, 1));
     }
   } else {
     cudaMemcpyAsync(b.F, b.S, nn * sizeof(double), cudaMemcpyDeviceToDevice, st);
@@ -849,9 +929,10 @@ cudaError_t set_big_attributes(int max_n) {
       cudaFuncSetAttribute(k_big_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, smem > 48 * 1024 ? smem : 48 * 1024);
   if (e != cudaSuccess) return e;
   const int smem_df = (int)big_solve_df_smem(max_n);
-  e = cudaFuncSetAttribute(k_big_solve_df, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           smem_df > 48 * 1024 ? smem_df : 48 * 1024);
-  if (e != cudaSuccess) return e;
+  for (const void* f : {(const void*)k_big_forward, (const void*)k_big_back}) {
+    e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_df > 48 * 1024 ? smem_df : 48 * 1024);
+    if (e != cudaSuccess) return e;
+  }
   return cudaFuncSetAttribute(k_big_update_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kUpdSmem);
 }
 
