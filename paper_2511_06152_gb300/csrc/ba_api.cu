@@ -1,6 +1,7 @@
 // Host side of the C ABI declared in include/ba.h: validation, the presort
 // that builds the deterministic reduction tables, device arenas, batch plans
 // with CUDA-graph replay, and the serving scheduler.
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <fstream>
@@ -334,11 +335,28 @@ cudaError_t scratch_alloc(ba_ctx* ctx, void** p, size_t bytes) {
   return cudaMallocFromPoolAsync(p, bytes, ctx->scratch, ctx->stream);
 }
 
-// Whether a kernel on the context's device may write doubles straight to p:
-// device memory of that device, aligned.
-bool direct_output(const ba_ctx* ctx, const double* p) {
-  if (!p) return true;
+// Whether a kernel on the context's device may write count doubles straight to
+// p: device memory of that device, aligned, all of it inside one allocation (a
+// shorter destination is left to the copies, which refuse it).
+bool direct_output(const ba_ctx* ctx, const double* p, size_t count) {
+  if (!p || count == 0) return true;
   if ((reinterpret_cast<uintptr_t>(p) & 7) != 0) return false;
+  using Range = CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr);
+  static const Range range = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q{};
+    if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      f = nullptr;
+    }
+    return reinterpret_cast<Range>(f);
+  }();
+  CUdeviceptr base = 0;
+  size_t size = 0;
+  const CUdeviceptr at = reinterpret_cast<CUdeviceptr>(p);
+  if (!range || range(&base, &size, at) != CUDA_SUCCESS || size - (size_t)(at - base) < sizeof(double) * count)
+    return false;
   cudaPointerAttributes a{};
   if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
     cudaGetLastError();
@@ -2873,7 +2891,8 @@ BA_API ba_status ba_get_state(ba_ctx* ctx, ba_cluster_id id, double* R, double* 
   const size_t total = nr + nt + nx;
   // device destinations the kernel can write itself get the state with no
   // block and no copies between
-  if (ptr_kind == BA_PTR_DEVICE && direct_output(ctx, R) && direct_output(ctx, T) && direct_output(ctx, X)) {
+  if (ptr_kind == BA_PTR_DEVICE && direct_output(ctx, R, nr) && direct_output(ctx, T, nt) &&
+      direct_output(ctx, X, nx)) {
     launch_export_state(c->d_desc, c->h, ctx->mixed, R, T, nx ? X : nullptr, ctx->stream);
     note_direct(ctx);
     CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
