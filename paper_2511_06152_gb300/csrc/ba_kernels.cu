@@ -907,7 +907,10 @@ __device__ __forceinline__ typename AccOf<Real>::T add_rows(const Real* part, in
 struct RedItem {
   const int* slots;
   const void* part;
-  int begin, n, width;  // n = 0: nothing to do (its cluster is inactive, or no such item)
+  // width = 0: nothing to do (its cluster is inactive, or no such item).  An empty
+  // list has n = 0 and its sums, zeros, are stored: a free image may observe
+  // nothing, and the arena holds whatever an earlier cluster left in it.
+  int begin, n, width;
   // lane e of the sums goes to out[(e / 6) ld + e % 6].  The pair block of a
   // cluster of up to kMaxFreeSmall free images goes negated to its place in the
   // lower triangle of S (elimination order; and mirrored to out2): where that
@@ -980,7 +983,7 @@ __global__ void __launch_bounds__(kRedThreads, 6) k_partial_reduce(BatchView bv,
     __syncthreads();
     if (seg < group) {  // the short lists, a group each
       const RedItem r = items[seg];
-      if (r.n > 0 && r.n <= kRedLong && el < abs(r.width)) {
+      if (r.n <= kRedLong && el < abs(r.width)) {
         const Real* part = (const Real*)r.part + red_element(r, el);
         const int stride = abs(r.width) == 36 ? kPairPart : kCamPart;
         red_store(r, el, add_rows<Real>(part, stride, r.slots, r.begin, r.begin + r.n).get());
