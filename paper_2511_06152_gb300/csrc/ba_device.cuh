@@ -35,7 +35,7 @@ __device__ __forceinline__ double recip_any(double x) {
   const double e = fma(-x, r, 1.0);
   return fma(r, fma(e, e, e), r);
 }
-// a > b for a constant b > 0 (false for NaN), on the bits: a binary64
+// a > b for b >= 0 (false for NaN), on the bits: a binary64
 // comparison occupies the binary64 pipe like a product
 __device__ __forceinline__ bool above(double a, double b) {
   const long long x = __double_as_longlong(a);
@@ -430,8 +430,11 @@ __device__ __forceinline__ void obs_step(const Real* Rm, Real dx, Real dy, Real 
   Real b0 = D00 * u0 + D01 * u1, b1 = D01 * u0 + D11 * u1;
   const Real a = f * iz;
   const Real m = front ? w * a * a : Real(0);
-  b0 *= m;
-  b1 *= m;
+  // A weight of zero selects zero: in binary32 b0 and b1 are infinite for a
+  // point 1e5 m beside an image and behind it (its coordinates enter to the
+  // tenth power), or where the squared error overflows, and 0 times that is NaN.
+  b0 = above(m, Real(0)) ? b0 * m : Real(0);
+  b1 = above(m, Real(0)) ? b1 * m : Real(0);
   const Real b2 = -(xn * b0 + yn * b1);
 #pragma unroll
   for (int i = 0; i < 3; ++i) g[i] = Rm[3 * i] * b0 + Rm[3 * i + 1] * b1 + Rm[3 * i + 2] * b2;
