@@ -428,6 +428,12 @@ __global__ void __launch_bounds__(256) k_big_split(const DevCluster* dcl) {
 constexpr int kPanelThreads = 1024;
 constexpr int kPld = kBigNB + 1;  // padded leading dimension of the shared blocks
 
+// 2^-floor(e / 2) of d = 2^e (1 .. 2)
+__device__ __forceinline__ float pow2_inv_sqrt(float d) {
+  const int e = ((__float_as_int(d) >> 23) & 0xff) - 127;
+  return __int_as_float((127 - (e >> 1)) << 23);
+}
+
 // Block column k: the diagonal block factored and inverted by every CTA
 // (double-float; rows past n padded with the identity), then CTA 0 stores
 // the inverse, CTA b (1 <= b <= m) the panel of row block k + b,
@@ -440,6 +446,13 @@ constexpr int kPld = kBigNB + 1;  // padded leading dimension of the shared bloc
 // the products to what is right of it; two barriers.  (The predecessor, a
 // column at a time with rank-pw updates by the whole CTA, took 22 k cycles of
 // the launch's 56 k; a sweep takes 1.2 k.)
+//
+// The block is scaled first, A' = E A E by powers of two with A'(i, i) in
+// [1, 4): the sweeps form products of two entries and reciprocals of pivots,
+// which leave the binary32 exponent range from entries of 2^64 on (a pixel sigma
+// of 1e-4 px).  L^-1 = L'^-1 E; the factors are powers of two, so inside
+// that range the results are the same bits with and without them (400 images,
+// three iterations, 8.53 and 8.56 ms).
 //
 // The right-hand side goes along as one more row of the matrix: every CTA takes
 // y_k = L_kk^-1 v_k, CTA 0 stores it and CTA b subtracts L_ik y_k from v_i: a
@@ -460,6 +473,7 @@ __global__ void __launch_bounds__(kPanelThreads) k_big_panel(const DevCluster* d
   __shared__ float Wh[kBigNB][kPld], Wl[kBigNB][kPld];           // inverse of the factor
   __shared__ float Ph[kBigNB][kPld], Pl[kBigNB][kPld];           // A_ik
   __shared__ dfl vk[kBigNB], yk[kBigNB];                          // the right-hand side's part
+  __shared__ float escale[kBigNB];                                // E
   __shared__ int s_fail;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int b = blockIdx.x;
@@ -478,6 +492,10 @@ __global__ void __launch_bounds__(kPanelThreads) k_big_panel(const DevCluster* d
     if (b > 0 && r < nr && c < nb) p = dfl{Fh[(size_t)(ri + r) * n + r0 + c], Fl[(size_t)(ri + r) * n + r0 + c]};
     if (tid < nb) w = fv[r0 + tid];
     if (!in && r == c) v.hi = 1.0f;
+    if (r == c) escale[c] = pow2_inv_sqrt(v.hi);
+    __syncthreads();
+    const float sr = escale[r], sc = escale[c];
+    v = dfl{v.hi * sr * sc, v.lo * sr * sc};
     *reinterpret_cast<dfl*>(blk(r >> 3, c >> 3) + elt_off(r & 7, c & 7)) = v;
     *reinterpret_cast<dfl*>(blk(kB + (r >> 3), c >> 3) + elt_off(r & 7, c & 7)) = dfl{r == c ? 1.0f : 0.0f, 0.0f};
     if (b > 0) {
@@ -527,13 +545,14 @@ __global__ void __launch_bounds__(kPanelThreads) k_big_panel(const DevCluster* d
       __syncthreads();
     }
   }
-  {  // inverse(r, c) = sqrt(d_r) l_c(r), r >= c
+  {  // inverse(r, c) = sqrt(d_r) l_c(r) s_c, r >= c
     const int r = tid >> 5, c = tid & 31;
+    const float sc = escale[c];
     dfl v{0.0f, 0.0f};
     if (c <= r)
       v = df_mul(*reinterpret_cast<const dfl*>(blk(kB + (c >> 3), r >> 3) + elt_off(c & 7, r & 7)), sq[r]);
-    Wh[r][c] = v.hi;
-    Wl[r][c] = v.lo;
+    Wh[r][c] = v.hi * sc;
+    Wl[r][c] = v.lo * sc;
   }
   __syncthreads();
   {  // y_k(r) = sum_q X(r, q) v_k(q): a warp per row
