@@ -116,9 +116,11 @@ __device__ __forceinline__ dfl df_recip(dfl b) {
   return fast_two_sum(r, __fmul_rn(r, e));
 }
 
-// the same from the hardware's approximate reciprocal, one binary32 Newton step
-// in place of the correctly rounded quotient (25 + 8 cycles instead of 84):
-// within an ulp of it before the double-float correction, which squares that
+// the same from the hardware's approximate reciprocal (documented within 2^-23):
+// one step of Newton's iteration for 1 / r = b squares its error below half an
+// ulp's rounding, in place of the correctly rounded quotient (25 + 8 cycles
+// instead of 84).  Over all 2^23 significands the result is no further from
+// 1 / b than df_recip's.
 __device__ __forceinline__ dfl df_recip_fast(dfl b) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(b.hi));
