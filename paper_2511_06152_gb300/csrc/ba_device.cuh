@@ -25,16 +25,7 @@ __device__ __forceinline__ float pivot_rsqrt(float d) {
   return d < 0x1p-100f ? rsqrtf(d * 0x1p100f) * 0x1p50f : rsqrtf(d);
 }
 __device__ __forceinline__ float recip_any(float x) { return __frcp_rn(x); }
-// 1 / x for a normal x from the hardware's approximation r (about 20 bits) by
-// the third-order Householder step r (1 + e + e^2), e = 1 - x r: three binary64
-// instructions of 64 cycles a warp where the quotient takes seven; the last,
-// a fused r + r (e + e^2), is the only rounding above 2^-60.
-__device__ __forceinline__ double recip_any(double x) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  const double e = fma(-x, r, 1.0);
-  return fma(r, fma(e, e, e), r);
-}
+__device__ __forceinline__ double recip_any(double x) { return 1.0 / x; }
 // a > b for b >= 0 (false for NaN), on the bits: a binary64
 // comparison occupies the binary64 pipe like a product
 __device__ __forceinline__ bool above(double a, double b) {

@@ -21,6 +21,11 @@ int on_device(const void* in, size_t in_bytes, void* out, size_t out_bytes, F la
   return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? 0 : 1;
 }
 
+__global__ void k_recip(const double* x, double* y, int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) y[i] = recip_any(x[i]);
+}
+
 // every binary32 significand, the low word from a hash of it: largest |b r - 1|
 // of the two reciprocals (in out[0] and out[1], as the bits of a binary64)
 __global__ void k_df_recip(float scale, unsigned long long* out) {
@@ -49,6 +54,11 @@ int grid(int n) { return (n + 127) / 128; }
 }  // namespace
 
 extern "C" {
+
+int probe_recip(const double* x, double* y, int n) {
+  return on_device(x, sizeof(double) * n, y, sizeof(double) * n,
+                   [&](char* a, char* b) { k_recip<<<grid(n), 128>>>((double*)a, (double*)b, n); });
+}
 
 int probe_df_recip(const float* scale, double* worst) {
   return on_device(scale, sizeof(float), worst, 2 * sizeof(double), [&](char*, char* b) {

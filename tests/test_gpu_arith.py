@@ -27,6 +27,16 @@ def _call(f, inp, out, *n):
     return out
 
 
+def test_binary64_reciprocal_is_the_quotient(probe):
+    """1 / z of the cost and the linearisation, from just above the smallest
+    depth (1e-6) on: the correctly rounded quotient, 0 for an infinite depth."""
+    rng = np.random.Generator(np.random.PCG64(1))
+    x = np.concatenate([np.nextafter(1e-6, 1.0) * (1 + rng.random(100_000)), 300.0 * (0.5 + rng.random(300_000)),
+                        np.ldexp(1 + rng.random(400_000), rng.integers(-20, 1023, 400_000)),
+                        2.0 - 2.0 ** -np.arange(1.0, 53.0), [np.inf]])
+    assert np.array_equal(_call(probe.probe_recip, x, np.empty_like(x), len(x)), 1.0 / x)
+
+
 @pytest.mark.parametrize("exponent", [-96, -37, 0, 1, 2])
 def test_pivot_reciprocal_is_as_accurate_as_the_quotients(probe, exponent):
     """1 / d of a pivot (double-float, Newton's iteration from the hardware's
