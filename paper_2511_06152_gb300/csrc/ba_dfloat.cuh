@@ -56,13 +56,6 @@ __device__ __forceinline__ dfl df_add(dfl a, dfl b) {
   return fast_two_sum(s.hi, s.lo);
 }
 
-// a + b rounded to binary32: the high words' sum exactly, the low words into
-// its remainder (within 2^-24 of an ulp of df_to_f(df_add(a, b)), at half its cost)
-__device__ __forceinline__ float df_sum_to_f(dfl a, dfl b) {
-  const dfl s = two_sum(a.hi, b.hi);
-  return __fadd_rn(s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo)));
-}
-
 // double-word + double-word, "sloppy" version (Dekker): the low words are
 // added without their own TwoSum.  Relative to max(|a|, |b|) the error stays
 // near 2^-44, but it is not relative to the result: only for sums without
@@ -185,6 +178,11 @@ __device__ __forceinline__ dfl df_rsqrt(dfl d) {
 }
 
 __device__ __forceinline__ float df_to_f(dfl a) { return __fadd_rn(a.hi, a.lo); }
+
+// a + b rounded to binary32.  The accurate sum: where the high words cancel (a
+// point and an image centre in grid coordinates), the low words' sum takes part
+// in full, and the result's only error is its own rounding.
+__device__ __forceinline__ float df_sum_to_f(dfl a, dfl b) { return df_add(a, b).hi; }
 __device__ __forceinline__ double df_to_d(dfl a) { return (double)a.hi + (double)a.lo; }
 
 // binary64 -> double-word (hi = rounded value, lo = rounded remainder)

@@ -26,6 +26,11 @@ __global__ void k_recip(const double* x, double* y, int n) {
   if (i < n) y[i] = recip_any(x[i]);
 }
 
+__global__ void k_sum(const dfl* ab, float* y, int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) y[i] = df_sum_to_f(ab[2 * i], ab[2 * i + 1]);
+}
+
 // every binary32 significand, the low word from a hash of it: largest |b r - 1|
 // of the two reciprocals (in out[0] and out[1], as the bits of a binary64)
 __global__ void k_df_recip(float scale, unsigned long long* out) {
@@ -58,6 +63,11 @@ extern "C" {
 int probe_recip(const double* x, double* y, int n) {
   return on_device(x, sizeof(double) * n, y, sizeof(double) * n,
                    [&](char* a, char* b) { k_recip<<<grid(n), 128>>>((double*)a, (double*)b, n); });
+}
+
+int probe_sum(const float* ab, float* y, int n) {
+  return on_device(ab, 4 * sizeof(float) * n, y, sizeof(float) * n,
+                   [&](char* a, char* b) { k_sum<<<grid(n), 128>>>((dfl*)a, (float*)b, n); });
 }
 
 int probe_df_recip(const float* scale, double* worst) {

@@ -37,6 +37,25 @@ def test_binary64_reciprocal_is_the_quotient(probe):
     assert np.array_equal(_call(probe.probe_recip, x, np.empty_like(x), len(x)), 1.0 / x)
 
 
+def test_difference_of_double_floats_rounds_once(probe):
+    """X - T of a point and an image centre in grid coordinates (5e5, 5e6 m),
+    1e-3 .. 1e3 m apart: rounded to binary32 from the exact difference.  The
+    accurate sum's relative error of 3 2^-48 is 3 2^-24 ulp of the result."""
+    rng = np.random.Generator(np.random.PCG64(2))
+    n = 1_000_000
+    X = np.where(rng.random(n) < 0.5, 5e5, 5e6) * (1 + 0.1 * rng.random(n))
+    T = X + 10.0 ** rng.uniform(-3, 3, n) * rng.choice([-1, 1], n)
+    ab = np.empty((n, 4), np.float32)
+    for i, v in ((0, X), (2, -T)):
+        ab[:, i] = v
+        ab[:, i + 1] = v - ab[:, i].astype(np.float64)
+    got = _call(probe.probe_sum, ab, np.empty(n, np.float32), n).astype(np.float64)
+    w = ab.astype(np.float64)  # both partial sums, and the total, are exact in binary64
+    exact = (w[:, 0] + w[:, 2]) + (w[:, 1] + w[:, 3])
+    ulp = np.spacing(np.abs(exact).astype(np.float32)).astype(np.float64)
+    assert (np.abs(got - exact) <= (0.5 + 2.0 ** -20) * ulp).all()
+
+
 @pytest.mark.parametrize("exponent", [-96, -37, 0, 1, 2])
 def test_pivot_reciprocal_is_as_accurate_as_the_quotients(probe, exponent):
     """1 / d of a pivot (double-float, Newton's iteration from the hardware's
