@@ -520,7 +520,8 @@ typedef struct {
   int32_t back_ctas_per_sm; /* back-substitution grid: CTAs per SM before it strides */
   int32_t factor_nb;        /* accepted and without effect: the factor of clusters of <= 32 free images works on
                                block columns of 8 */
-  int32_t factor_threads;   /* that factor runs on four CTAs of half as many threads (at least 192) */
+  int32_t factor_threads;   /* that factor runs on four CTAs of half as many threads (at least 192: 256 and 384
+                               are the same) */
   int32_t big_panel_w;      /* accepted and without effect: that solver's diagonal blocks go in blocks of 8 */
   int32_t batch_chains;     /* a batch's LM iterations as this many concurrent launch chains over disjoint
                                parts of the batch (clusters dealt by decreasing size); 1: one chain */
@@ -544,8 +545,11 @@ BA_API ba_status ba_set_tune(ba_ctx* ctx, const ba_tune* t);
  * initial state), and timed with CUDA events on the context's stream, the
  * fastest of three solves per candidate; one parameter at a time, each over
  * a few candidates around the current choice, in the order above (a
- * coordinate descent from the defaults).  The choice is kept in the context and written
- * to *out with both timings; the tuning clusters are destroyed.  Blocking;
+ * coordinate descent from the defaults, with one chunk size for all
+ * clusters).  Where the defaults, whose chunk size goes by the cluster, are
+ * faster than the result, they are the choice (chunk_tiles 0).  The choice is
+ * kept in the context and written to *out with both timings; the tuning
+ * clusters are destroyed.  Blocking;
  * takes seconds (chunk_tiles candidates re-create the clusters).
  * BA_ERR_INVALID for bad arguments or while a cluster is in service; errors
  * of cluster creation are returned as they come. */

@@ -365,13 +365,15 @@ bool direct_output(const ba_ctx* ctx, const double* p, size_t count) {
   return a.type == cudaMemoryTypeDevice && a.device == ctx->device;
 }
 
+constexpr int kMinChunkTiles = 4;  // the smallest chunk size that can be set
+
 bool tune_in_range(const ba_tune& t, bool mixed, std::string* why) {
   const int cmax = chunk_tiles(mixed);
   auto bad = [&](const char* m) {
     *why = m;
     return false;
   };
-  if (t.chunk_tiles != 0 && (t.chunk_tiles < 4 || t.chunk_tiles > cmax))
+  if (t.chunk_tiles != 0 && (t.chunk_tiles < kMinChunkTiles || t.chunk_tiles > cmax))
     return bad("chunk_tiles must be 0 or 4 .. 16 (mixed) / 8 (FP64)");
   if (t.lin_ctas_per_sm < 1 || t.lin_ctas_per_sm > 32) return bad("lin_ctas_per_sm must be 1 .. 32");
   if (t.back_ctas_per_sm < 1 || t.back_ctas_per_sm > 32) return bad("back_ctas_per_sm must be 1 .. 32");
@@ -3089,8 +3091,7 @@ BA_API ba_status ba_autotune(ba_ctx* ctx, const ba_cluster_desc* descs, int32_t 
     ba_tune bt = tune_to_abi(t);
     ba_status st = ba_set_tune(ctx, &bt);
     if (st != BA_OK) return st;
-    const int ct = t.chunk_tiles > 0 ? t.chunk_tiles : chunk_tiles(ctx->mixed);
-    if (ct != created) {
+    if (t.chunk_tiles != created) {
       destroy_all();
       for (int i = 0; i < n; ++i) {
         ba_cluster_id id = 0;
@@ -3098,7 +3099,7 @@ BA_API ba_status ba_autotune(ba_ctx* ctx, const ba_cluster_desc* descs, int32_t 
         if (st != BA_OK) return st;
         ids.push_back(id);
       }
-      created = ct;
+      created = t.chunk_tiles;
     }
     double best = 1e300;
     for (int rep = 0; rep < 4; ++rep) {
@@ -3116,12 +3117,32 @@ BA_API ba_status ba_autotune(ba_ctx* ctx, const ba_cluster_desc* descs, int32_t 
     *ms = best;
     return BA_OK;
   };
-  TuneParams cur;  // the defaults
-  cur.chunk_tiles = chunk_tiles(ctx->mixed);
-  double cur_ms = 0.0;
-  ba_status st = measure(cur, &cur_ms);
+  double ms_default = 0.0;
+  ba_status st = measure(TuneParams{}, &ms_default);
   if (st != BA_OK) return finish(st);
-  const double ms_default = cur_ms;
+  // The search goes over explicit chunk sizes.  It starts from the one that the
+  // default gives the clusters where that is the same for all of them (and can
+  // be set), else from the largest.
+  TuneParams cur;
+  {
+    std::lock_guard<std::mutex> g(ctx->api_mu);
+    for (size_t i = 0; i < ids.size(); ++i) {
+      const Cluster* c = find_cluster(ctx, ids[i]);
+      const int ct = c ? default_chunk_tiles(c->h.n_tiles, c->nf, ctx->mixed) : 0;
+      cur.chunk_tiles = i == 0 || ct == cur.chunk_tiles ? ct : 0;
+      if (cur.chunk_tiles < kMinChunkTiles) {
+        cur.chunk_tiles = 0;
+        break;
+      }
+    }
+  }
+  double cur_ms = ms_default;
+  if (cur.chunk_tiles > 0) {  // the clusters and launches just measured
+    created = cur.chunk_tiles;
+  } else {
+    cur.chunk_tiles = chunk_tiles(ctx->mixed);
+    if ((st = measure(cur, &cur_ms)) != BA_OK) return finish(st);
+  }
   // one parameter at a time; a candidate replaces the current value only
   // when it is faster by more than 1 % (timing noise keeps the default)
   struct Knob {
@@ -3130,16 +3151,17 @@ BA_API ba_status ba_autotune(ba_ctx* ctx, const ba_cluster_desc* descs, int32_t 
   };
   const bool mixed = ctx->mixed;
   const std::vector<Knob> knobs = {
-      {&TuneParams::chunk_tiles, mixed ? std::vector<int>{12, 8} : std::vector<int>{6, 4}},
+      {&TuneParams::chunk_tiles, mixed ? std::vector<int>{16, 12, 8, 4} : std::vector<int>{8, 6, 4}},
       {&TuneParams::lin_ctas_per_sm, {4, 2}},
       {&TuneParams::back_ctas_per_sm, {8, 4}},
-      {&TuneParams::factor_threads, {384, 256}},
+      {&TuneParams::factor_threads, {384}},  // (256 launches the same)
       {&TuneParams::batch_chains, {2, 8}},
   };
   for (const Knob& k : knobs) {
     TuneParams best = cur;
     double best_ms = cur_ms;
     for (int v : k.cands) {
+      if (v == cur.*(k.field)) continue;
       TuneParams t = cur;
       t.*(k.field) = v;
       double ms = 0.0;
@@ -3152,6 +3174,10 @@ BA_API ba_status ba_autotune(ba_ctx* ctx, const ba_cluster_desc* descs, int32_t 
     }
     cur = best;
     cur_ms = best_ms;
+  }
+  if (ms_default < cur_ms) {  // sizes by cluster beat any one size
+    cur = TuneParams{};
+    cur_ms = ms_default;
   }
   ba_tune bt = tune_to_abi(cur);
   st = ba_set_tune(ctx, &bt);
