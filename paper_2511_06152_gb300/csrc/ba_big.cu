@@ -1,7 +1,7 @@
 // Reduced camera systems larger than one CTA's shared memory holds (more than
 // kMaxFreeSmall free images, n = 6 n_free > 192; the 400-image large block
 // has n = 2400), solved in global memory.  Same system and elimination order
-// as the shared-memory solver of ba_kernels.cu: S assembled in binary64 in
+// as the shared-memory solver of ba_factor.cu: S assembled in binary64 in
 // the reverse Cuthill-McKee order, Cholesky restricted to the envelope of S
 // (no fill outside it), a solve, refinement steps against S in binary64.
 //
@@ -383,8 +383,6 @@ __device__ __forceinline__ float* df_lo(const DevCluster& C) {
   return reinterpret_cast<float*>(C.F) + (size_t)n * n;
 }
 
-// F = S on the lower triangle as double-float (entries outside the envelope
-// are zero in S and become zero here), one CTA per row.
 // The forward substitution's vectors on the tensor-core path, n double-floats
 // each in bx: v (the right-hand side less what the block columns done so far
 // take off it) and y = L^-1 rhs.
@@ -401,6 +399,8 @@ __device__ __forceinline__ Dot2 warp_merge(Dot2 d, int width) {
   return d;
 }
 
+// F = S on the lower triangle as double-float (entries outside the envelope
+// are zero in S and become zero here), one CTA per row; v = rhs.
 __global__ void __launch_bounds__(256) k_big_split(const DevCluster* dcl) {
   dependency_wait();
   dependency_trigger();

@@ -33,7 +33,7 @@ constexpr int kChunkObsMixed = 32 * kChunkTilesMixed;  // at most this many obse
 constexpr int kChunkObsF64 = 32 * kChunkTilesF64;
 constexpr int kChunkThreads = 256;
 constexpr int kMaxTrack = 32;
-constexpr int kMaxFreeSmall = 32;  // free cameras the single-CTA factor handles (n <= 192)
+constexpr int kMaxFreeSmall = 32;  // free cameras the shared-memory factor handles (n <= 192)
 constexpr int kMaxBatchChains = 8;  // concurrent launch chains of a batch's LM iterations, at most
 constexpr int kMaxFree = 1024;     // free cameras of one cluster (larger systems: the global-memory solver)
 constexpr int kBigNB = 32;         // block size of the global-memory factorisation
@@ -98,8 +98,8 @@ struct LmState {
   float mu_f;        // mu rounded to binary32 (mixed-path kernels)
   int needs_init;    // F must be evaluated at the current state before the next iteration
   int dev_error;     // a kernel gave up on a bounded wait this iteration (kDevErrTimeout); rejects the step
-  int tiles_done;    // back-substitution tiles finished this iteration; the warp that finishes the last
-                     // one takes the cluster's LM decision (zeroed by the factor kernels)
+  int tiles_done;    // back-substitution tiles finished this iteration; the CTA of the warp that finishes the
+                     // last one takes the cluster's LM decision (zeroed by the factor kernels)
   int iter0;         // iter when the cluster was last armed
   double ftol;       // serving: an accepted step after the first that lowers F by at most ftol * F
                      // ends the solve (0: off)
@@ -159,9 +159,9 @@ struct DevCluster {
   float* camdf;            // mixed path: [2][nc][kCamDf] double-float cameras
 
   // per point, from the current iteration's linearisation: M = L^-1 of the
-  // damped point block (m00 m10 m11 m20 m21 m22), q = M g_p, D_p, g_p, pad;
-  // Real [n_pts][16], written by the linearise+Schur kernel for the
-  // back-substitution
+  // damped point block (m00 m10 m11 m20 m21 m22), q = M g_p (read by no kernel),
+  // D_p, g_p, pad; Real [n_pts][16], written by the linearise+Schur kernel for
+  // the back-substitution
   void* ptblk;
   const Tile* tiles;       // [n_tiles]
   const int* obs_cam;      // [no] point-major
@@ -380,6 +380,8 @@ int chunk_tiles(bool mixed);
 // iteration in chunks of 8, 32 in chunks of 2.  Clusters of more than
 // kMaxFreeSmall free images, whose iteration is the global-memory solver's,
 // keep the maximum: their chunks hold more image pairs the smaller they are.
+// 152 is the SM count of a GB300, written out because the presort that builds
+// the chunks also runs without a device.
 inline int default_chunk_tiles(int n_tiles, int n_free, bool mixed) {
   int t = n_free > kMaxFreeSmall ? kChunkTilesF64 : (n_tiles + 151) / 152;
   t = t < 2 ? 2 : (t > kChunkTilesF64 ? kChunkTilesF64 : t);

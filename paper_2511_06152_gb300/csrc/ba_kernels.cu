@@ -13,17 +13,20 @@
 //                    co-visible image pair the sum of Z_a Z_b^T, each job on a
 //                    run of lanes sized by its cost.  One partial sum per job.
 //   k_partial_reduce the chunks' partial sums of each image and each pair,
-//                    added in chunk order (FP64).
-//   k_factor_solve   per cluster (FP64): assemble S = U* - W V*^-1 W^T and
-//                    rhs = g_c - W V*^-1 g_p with priors and damping, blocked
-//                    Cholesky in shared memory, solve, iterative refinement,
-//                    candidate camera poses.  (Clusters of more than 32 free
-//                    images: the global-memory solver of ba_big.cu.)
-//   k_backsub_cost   per tile: linearise again (same arithmetic, same values),
-//                    dX = M^T (q - sum_k Z_k^T dc_k), candidate points, cost
-//                    at the candidate and the predicted reduction; the warp
-//                    that finishes a cluster's last tile takes its LM step:
-//                    gain ratio, accept/reject, Nielsen update.
+//                    added in a fixed order; the pair sums go to their places
+//                    in S.
+//   k_factor_solve   per cluster (ba_factor.cu): assemble S = U* - W V*^-1 W^T
+//                    and rhs = g_c - W V*^-1 g_p with priors and damping,
+//                    L D L^T in the shared memory of four CTAs, solve,
+//                    iterative refinement, candidate camera poses.  (Clusters
+//                    of more than 32 free images: the global-memory solver of
+//                    ba_big.cu.)
+//   k_backsub_cost   per tile: each observation's Jp^T (Jc dc) from its image's
+//                    step, without Jacobians; dX = M^T M (g_p - their sum),
+//                    candidate points, cost at the candidate and the predicted
+//                    reduction; the CTA whose warp finishes a cluster's last
+//                    tile takes its LM step: gain ratio, accept/reject, Nielsen
+//                    update.
 //   Four launches per LM iteration.
 //
 // Precision.  MIXED = false: every step in binary64.  MIXED = true: the
@@ -35,7 +38,7 @@
 //
 // Every sum runs in an order fixed by the cluster's presorted tables; the
 // only atomic is the back-substitution's per-cluster tile counter, which
-// chooses the warp that takes the LM step and enters no sum.
+// chooses the CTA that takes the LM step and enters no sum.
 #include <cuda_runtime.h>
 #include <stdio.h>
 
@@ -855,7 +858,8 @@ __device__ __forceinline__ AccF acc_join(AccF a, AccF b) { return AccF{df_add(a.
 __device__ __forceinline__ AccD acc_join(AccD a, AccD b) { return AccD{a.v + b.v}; }
 
 // Every free camera and camera pair ("item") of the batch's clusters: its
-// chunk partials, added, into camsum / pairsum.
+// chunk partials, added, into camsum, and into S (pairsum for the
+// global-memory solver).
 //
 // Per iteration on GB300: one cluster of 235 k observations 39 -> 12 us (97 ->
 // 19 in binary64), 12 clusters 25 -> 21, 128 clusters 68 -> 83: their short
@@ -1015,9 +1019,9 @@ __global__ void __launch_bounds__(kRedThreads, 6) k_partial_reduce(BatchView bv,
 
 // ------------------------------------------------------------------ K5
 
-// Back-substitution and candidate cost, warp per tile.  The tile is
-// linearised again (the same arithmetic as in k_lin_schur) instead of reading
-// per-observation records back from memory.
+// Back-substitution and candidate cost, warp per tile.  Each observation's
+// products are formed again from its image's step (obs_step, no Jacobians)
+// instead of reading per-observation records back from memory.
 template <bool MIXED>
 __device__ void backsub_tile(const DevCluster& C, LmState* lm, int local, int lane);
 
@@ -1275,35 +1279,6 @@ __global__ void __launch_bounds__(256) k_cost_tiles(BatchView bv) {
 }
 
 // fixed-order block sum of tilepart[:, which]
-// Both per-tile sums (cost at the candidate, pred) over the cluster's tiles,
-// in a fixed order: each thread a strided run of tiles, then a warp tree and
-// the warps in order.  red: shared [2][blockDim / 32].  Valid in thread 0.
-__device__ double2 block_sum_tiles2(const DevCluster& C, double* red) {
-  double a = 0.0, b = 0.0;
-  const double2* tp = reinterpret_cast<const double2*>(C.tilepart);
-  for (int i = threadIdx.x; i < C.n_tiles; i += blockDim.x) {
-    const double2 v = tp[i];
-    a += v.x;
-    b += v.y;
-  }
-  a = warp_sum(a);
-  b = warp_sum(b);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  if (lane == 0) {
-    red[wid] = a;
-    red[nw + wid] = b;
-  }
-  __syncthreads();
-  double2 tot = make_double2(0.0, 0.0);
-  if (threadIdx.x == 0)
-    for (int w = 0; w < nw; ++w) {
-      tot.x += red[w];
-      tot.y += red[nw + w];
-    }
-  __syncthreads();
-  return tot;
-}
-
 __device__ double block_sum_tiles(const DevCluster& C, int which, double* red) {
   double v = 0.0;
   for (int i = threadIdx.x; i < C.n_tiles; i += blockDim.x) v += C.tilepart[2 * i + which];
