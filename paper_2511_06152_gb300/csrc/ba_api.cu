@@ -149,8 +149,7 @@ struct ba_ctx {
   std::atomic<uint64_t> launches{0};
   std::mutex api_mu;  // cluster table, plans, budget; never held across a serving round
   cudaMemPool_t pool = nullptr;  // device memory of clusters and plans (stream-ordered)
-  cudaMemPool_t scratch = nullptr;  // device scratch of single calls, made by the first (scratch_alloc)
-  std::mutex scratch_mu;
+  cudaMemPool_t scratch = nullptr;  // device scratch of single calls (scratch_alloc)
 
   // serving
   std::mutex sv_mu;
@@ -325,39 +324,14 @@ cudaError_t pool_alloc(ba_ctx* ctx, void** p, size_t bytes, cudaStream_t st) {
   return cudaMallocFromPoolAsync(p, bytes, ctx->pool, st);
 }
 
-cudaMemPoolProps device_pool_props(int device) {
-  cudaMemPoolProps props{};
-  props.allocType = cudaMemAllocationTypePinned;
-  props.location.type = cudaMemLocationTypeDevice;
-  props.location.id = device;
-  return props;
-}
-
 // Device scratch of one call, on the context's stream, from a pool of its own
 // that keeps up to kScratchKeep bytes between calls.  The device's default pool
 // gives its memory back at every synchronisation, so that each call mapped it
 // anew: ba_get_state of one cluster took 290 us, of which its kernel and copies
 // are 20.  Apart from the clusters' pool, so that no creation is handed (and
-// ordered behind) memory a solve's stream still uses.  Made by the first call
-// that needs it: a context opens in 40 us without it, in 65 with it.
+// ordered behind) memory a solve's stream still uses.
 constexpr uint64_t kScratchKeep = (uint64_t)64 << 20;
 cudaError_t scratch_alloc(ba_ctx* ctx, void** p, size_t bytes) {
-  {
-    std::lock_guard<std::mutex> g(ctx->scratch_mu);
-    if (!ctx->scratch) {
-      cudaMemPoolProps props = device_pool_props(ctx->device);
-      uint64_t keep = kScratchKeep;
-      cudaMemPool_t pool = nullptr;
-      cudaError_t e = cudaMemPoolCreate(&pool, &props);
-      if (e != cudaSuccess) return e;
-      e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
-      if (e != cudaSuccess) {
-        cudaMemPoolDestroy(pool);
-        return e;
-      }
-      ctx->scratch = pool;
-    }
-  }
   return cudaMallocFromPoolAsync(p, bytes, ctx->scratch, ctx->stream);
 }
 
@@ -2428,14 +2402,20 @@ BA_API ba_status ba_init(ba_ctx** out, const ba_config* cfg) {
     }
     ctx->own_stream = true;
   }
-  const cudaMemPoolProps props = device_pool_props(cfg->device);
-  const uint64_t keep = UINT64_MAX;
+  cudaMemPoolProps props{};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = cfg->device;
+  const uint64_t keep = UINT64_MAX, keep_scratch = kScratchKeep;
   if (cudaStreamCreateWithFlags(&ctx->sched_stream, cudaStreamNonBlocking) != cudaSuccess ||
       cudaStreamCreateWithFlags(&ctx->plan_stream, cudaStreamNonBlocking) != cudaSuccess ||
       cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking) != cudaSuccess ||
       cudaMemPoolCreate(&ctx->pool, &props) != cudaSuccess ||
-      cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, (void*)&keep) != cudaSuccess) {
+      cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, (void*)&keep) != cudaSuccess ||
+      cudaMemPoolCreate(&ctx->scratch, &props) != cudaSuccess ||
+      cudaMemPoolSetAttribute(ctx->scratch, cudaMemPoolAttrReleaseThreshold, (void*)&keep_scratch) != cudaSuccess) {
     if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
+    if (ctx->scratch) cudaMemPoolDestroy(ctx->scratch);
     if (ctx->sched_stream) cudaStreamDestroy(ctx->sched_stream);
     if (ctx->plan_stream) cudaStreamDestroy(ctx->plan_stream);
     if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
@@ -3328,7 +3308,7 @@ BA_API ba_status ba_shutdown(ba_ctx* ctx) {
   }
   cudaStreamSynchronize(ctx->stream);
   cudaMemPoolDestroy(ctx->pool);
-  if (ctx->scratch) cudaMemPoolDestroy(ctx->scratch);
+  cudaMemPoolDestroy(ctx->scratch);
   cudaStreamDestroy(ctx->sched_stream);
   cudaStreamDestroy(ctx->plan_stream);
   cudaStreamDestroy(ctx->copy_stream);
