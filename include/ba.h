@@ -88,7 +88,9 @@ typedef uint64_t ba_ticket;     /* 0 is never a valid ticket */
 typedef struct {
   int32_t device;            /* CUDA device ordinal */
   void* stream;              /* cudaStream_t to run on; NULL: the library creates one */
-  uint64_t hbm_budget_bytes; /* device memory the context may hold; 0 = unlimited */
+  uint64_t hbm_budget_bytes; /* device memory of clusters and plans the context may hold; 0 = unlimited.  Beside it,
+                              * the scratch of single calls (read-back, footprints, patch transfer, traces): up to
+                              * 64 MiB of it stays with the context between calls */
   int32_t precision;         /* BA_FP64 or BA_MIXED */
   int32_t n_slots;           /* clusters the serving scheduler runs at once (ba_submit); 0 = 64 */
   int32_t refine_steps;      /* iterative-refinement passes against the binary64 S after the Cholesky

@@ -329,7 +329,11 @@ cudaError_t pool_alloc(ba_ctx* ctx, void** p, size_t bytes, cudaStream_t st) {
 // gives its memory back at every synchronisation, so that each call mapped it
 // anew: ba_get_state of one cluster took 290 us, of which its kernel and copies
 // are 20.  Apart from the clusters' pool, so that no creation is handed (and
-// ordered behind) memory a solve's stream still uses.
+// ordered behind) memory a solve's stream still uses.  Made with the context,
+// which opens in 65 us instead of 40 for it; a context that is opened, creates,
+// solves and reads back one small cluster and is closed takes 1.19 ms instead
+// of 1.50.  (Made by the first call that needs it, that call takes 25 to 60 us
+// more.)
 constexpr uint64_t kScratchKeep = (uint64_t)64 << 20;
 cudaError_t scratch_alloc(ba_ctx* ctx, void** p, size_t bytes) {
   return cudaMallocFromPoolAsync(p, bytes, ctx->scratch, ctx->stream);
