@@ -549,7 +549,8 @@ BA_API ba_status ba_set_tune(ba_ctx* ctx, const ba_tune* t);
  * a few candidates around the current choice, in the order above (a
  * coordinate descent from the defaults, with one chunk size for all
  * clusters).  Where the defaults, whose chunk size goes by the cluster, are
- * faster than the result, they are the choice (chunk_tiles 0).  The choice is
+ * faster than the result (the two timed again in turn where they are close),
+ * they are the choice (chunk_tiles 0).  The choice is
  * kept in the context and written to *out with both timings; the tuning
  * clusters are destroyed.  Blocking;
  * takes seconds (chunk_tiles candidates re-create the clusters).
